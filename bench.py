@@ -386,7 +386,7 @@ def measure_single(wl: Workload, steps: int, warmup: int, barrier=local_barrier,
         ms, reps = timed_repeats(s.step, stream, steps, barrier)
         flags = s.status()
         mass = s.mass()
-    out = {"ms": ms, "repeats_ms": reps, "status_flags": flags,
+    out = {"ms": ms, "repeats_ms": reps, "status_flags": flags, "launches": s.step_launches(steps),
            "mass_drift_rel": float(np.max(np.abs(mass - mass0) / np.abs(mass0))),
            "x0_host": x0_host, "stream": stream}
     if keep:
@@ -441,7 +441,7 @@ def single_line(wl: Workload, m: dict, steps: int, world: int, t_ms: float, sms:
                   % (state_gb * 1e3)),
         },
         "roofline": roof,
-        "gpu_launches": steps,
+        "gpu_launches": m.get("launches", steps),
         "status_flags": m["status_flags"],
         "mass_drift_rel": m["mass_drift_rel"],
     }

@@ -345,6 +345,11 @@ int lbms_adjoint_reduce(lbms_t* h, const void* gacc, double* dL_dD);
 /* Number of steps taken since lbms_set_state, or -1 for a NULL handle. */
 long lbms_steps_done(const lbms_t* h);
 
+/* Kernel launches that lbms_step(h, n_steps) makes (or replays): grids beyond the
+ * L2 cache take several steps per launch on the 1D and 2D lattices in F32.  0 for
+ * n_steps < 1, -1 for a NULL handle. */
+long lbms_step_launches(const lbms_t* h, long n_steps);
+
 /* Device address, inside the caller's workspace, of the buffer that holds the
  * current post-collision populations (layout as lbms_get_state).  It changes
  * with every step (the two buffers alternate) and after lbms_set_state_raw;

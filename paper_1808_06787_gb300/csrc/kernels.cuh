@@ -342,12 +342,12 @@ __device__ __forceinline__ void load_pair_y(const T* __restrict__ fin, uint32_t 
 // full-size grids: for D1Q3, D2Q4, D2Q5 and D3Q6 (ternary) the largest count at
 // which the plain step compiles without spilling (40, 40, 48 and 56
 // registers), each faster than fewer blocks while one more (spilling) is
-// slower; for D3Q7, 9 blocks at 56 registers with a 24-byte spill (0.3 %
-// faster than 8 blocks without; 10 blocks, 48 registers: 2 % slower).
+// slower; for D3Q7, 8 blocks (256^3: 263.9 us per step; 7: 264.4, 9 with a spill:
+// 268.1, 10: 269.2).
 template <int LAT, int S, typename T>
 struct PairOccupancy {
     static constexpr int Q = Lattice<LAT>::Q;
-    static constexpr int value = S <= 1 ? 12 : (Q <= 4 ? 12 : (Q == 5 ? 10 : 9));
+    static constexpr int value = S <= 1 ? 12 : (Q <= 4 ? 12 : (Q == 5 ? 10 : (Q == 6 ? 9 : 8)));
     // the mass-writing variant holds the pair's mole fractions too: on the 3D
     // lattices it keeps 8 blocks (D3Q7 at 64 registers spills 28 bytes instead
     // of 68; 20-step calls 1.042 -> 1.044 of the copy peak)

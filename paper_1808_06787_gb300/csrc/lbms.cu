@@ -218,6 +218,8 @@ struct lbms_s {
     int nx = 1, ny = 1, nz = 1;
     uint32_t cells = 0, blocks = 0;  // blocks: of the step and mass kernels (mass partial slots)
     uint32_t step_block = 256;        // their threads per block
+    int sms = 1;                      // multiprocessors of the device
+    int depth = 1;                    // most plain steps one launch takes (fused_depth)
     uint32_t noflux = 0;
     uint32_t dirichlet = 0;  // Dirichlet faces
     uint32_t halo = 0;       // slab cut faces (LBMS_HALO)
@@ -323,6 +325,7 @@ KArgs base_args(const lbms_t* h, cudaStream_t st)
     memcpy(a.xref, h->xref, sizeof(a.xref));
     a.status = h->status;
     a.fixed_shift = h->fixed_shift;
+    a.sms = h->sms;
     a.stream = st;
     return a;
 }
@@ -344,6 +347,35 @@ cudaError_t launch_step(const lbms_t* h, int src, bool mass, cudaStream_t st)
     return dispatch(h, mass ? OP_STEP_MASS : OP_STEP, a);
 }
 
+// `m` plain steps from f[src] into f[1 - src] in one pass (2 <= m <= h->depth).
+cudaError_t launch_fused_steps(const lbms_t* h, int src, int m, cudaStream_t st)
+{
+    KArgs a = base_args(h, st);
+    a.fin = h->f[src];
+    a.fout = h->f[1 - src];
+    a.clock_in = h->clock + src;
+    a.clock_out = h->clock + (1 - src);
+    a.steps = m;
+    return dispatch_fused(h->lattice, a);
+}
+
+// Launches a run of n plain steps takes: passes of at most h->depth steps.
+long plain_launches(const lbms_t* h, long n) { return (n + h->depth - 1) / h->depth; }
+
+// n plain steps from f[src], split evenly over the passes (so that none is left a
+// single step where it can be helped); src becomes the buffer that holds the result.
+cudaError_t launch_plain(const lbms_t* h, int& src, long n, cudaStream_t st)
+{
+    for (long passes = plain_launches(h, n); passes > 0; --passes) {
+        const int m = (int)((n + passes - 1) / passes);
+        cudaError_t e = m == 1 ? launch_step(h, src, false, st) : launch_fused_steps(h, src, m, st);
+        if (e != cudaSuccess) return e;
+        src = 1 - src;
+        n -= m;
+    }
+    return cudaSuccess;
+}
+
 cudaError_t launch_finalize(const lbms_t* h, cudaStream_t st)
 {
     if (h->dtype == LBMS_F32)
@@ -355,7 +387,26 @@ cudaError_t launch_finalize(const lbms_t* h, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// Capture kGraphSteps plain steps starting from buffer `parity`.
+// Most steps one launch takes (fused.cuh): the lattice's limit on grids where a pass over
+// several steps beats as many single steps.  Same-box times of 60-step calls, single ->
+// fused: D2Q5 ternary 1448^2 27.6 -> 24.9 us per step, 1024^2 14.0 -> 13.7 and 4096 x 300
+// 16.1 -> 16.2 (hence the higher line for it), 4096^2 194 -> 138; binary 1024^2 8.4 -> 6.0;
+// D2Q9 ternary 1024^2 23.1 -> 18.8, 724^2 11.1 -> 14.5; five species 724^2 24.3 -> 21.2;
+// lines at every length (10^4 nodes 1.80 -> 0.86, 10^6 9.6 -> 5.0).  Planes narrower than
+// two strips or lower than a few parts keep single steps, and so do grids whose planes
+// exceed 32-bit byte offsets.
+int fused_depth(const lbms_t* h)
+{
+    if (h->dtype != LBMS_F32 || h->relax == LBMS_RELAX_FROZEN || h->dirichlet || h->halo) return 1;
+    if (h->cells >= (1u << 30)) return 1;
+    if (h->dim == 2) {
+        if (h->nx < 56 || h->ny < 24) return 1;
+        const uint32_t least = h->S >= 3 ? 1u << 19 : (h->S == 2 && h->Q <= 5 ? 3u << 19 : 1u << 20);
+        if (h->cells < least) return 1;
+    }
+    return fused_limit_of(h->lattice, h->n);
+}
+
 // The captured graphs hold the kernel arguments: dropped whenever those change.
 void drop_graphs(lbms_t* h)
 {
@@ -376,12 +427,9 @@ cudaError_t build_call_graph(lbms_t* h, long n, int parity, cudaGraphExec_t* out
 {
     cudaError_t e = cudaStreamBeginCapture(h->capture, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
-    cudaError_t le = cudaSuccess;
     int src = parity;
-    for (long i = 0; i < n && le == cudaSuccess; ++i) {
-        le = launch_step(h, src, i == n - 1, h->capture);
-        src = 1 - src;
-    }
+    cudaError_t le = launch_plain(h, src, n - 1, h->capture);
+    if (le == cudaSuccess) le = launch_step(h, src, true, h->capture);
     cudaGraph_t g = nullptr;
     e = cudaStreamEndCapture(h->capture, &g);
     if (le != cudaSuccess) {
@@ -424,12 +472,8 @@ cudaError_t build_graph(lbms_t* h, int parity, int j)
 {
     cudaError_t e = cudaStreamBeginCapture(h->capture, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
-    cudaError_t le = cudaSuccess;
     int src = parity;
-    for (int i = 0; i < kGraphLens[j] && le == cudaSuccess; ++i) {
-        le = launch_step(h, src, false, h->capture);
-        src = 1 - src;
-    }
+    cudaError_t le = launch_plain(h, src, kGraphLens[j], h->capture);
     cudaGraph_t g = nullptr;
     e = cudaStreamEndCapture(h->capture, &g);
     if (le != cudaSuccess) {
@@ -585,11 +629,13 @@ int lbms_create(lbms_t** out, int lattice, int n_species, const int grid[3], con
     h->cells = (uint32_t)((size_t)grid[0] * grid[1] * grid[2]);
     h->blocks = step_blocks(h->cells, sms);
     h->step_block = step_block_for(h->cells, sms);
+    h->sms = sms;
     h->noflux = noflux;
     h->dirichlet = dirichlet;
     h->halo = halo;
     h->plane = (uint32_t)split_plane(lattice, grid);
     h->es = dtype == LBMS_F64 ? 8 : 4;
+    h->depth = fused_depth(h);
     for (int i = 0; i < n; ++i)
         for (int j = 0; j < n; ++j) h->invD[i][j] = i == j ? 0.0 : 1.0 / D[i * n + j];
     h->ws = static_cast<char*>(workspace);
@@ -743,7 +789,7 @@ int lbms_step(lbms_t* h, long n_steps)
         if (g) {
             e = cudaGraphLaunch(g, h->stream);
             if (e != cudaSuccess) return cuda_fail(h, e, "cudaGraphLaunch");
-            if (n_steps & 1) h->cur = 1 - h->cur;
+            if ((plain_launches(h, n_steps - 1) + 1) & 1) h->cur = 1 - h->cur;
             h->steps += n_steps;
             h->partials_valid = true;
             h->mass_valid = false;
@@ -764,17 +810,18 @@ int lbms_step(lbms_t* h, long n_steps)
             }
             e = cudaGraphLaunch(h->graph[h->cur][j], h->stream);
             if (e != cudaSuccess) return cuda_fail(h, e, "cudaGraphLaunch");
+            if (plain_launches(h, kGraphLens[j]) & 1) h->cur = 1 - h->cur;
             left -= kGraphLens[j];
             h->steps += kGraphLens[j];
         }
         if (!h->graphs_ok) break;
     }
     while (left > 1) {
-        e = launch_step(h, h->cur, false, h->stream);
+        const long m = left - 1 < kCallGraphMax ? left - 1 : kCallGraphMax;
+        e = launch_plain(h, h->cur, m, h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "step kernel");
-        h->cur = 1 - h->cur;
-        --left;
-        ++h->steps;
+        left -= m;
+        h->steps += m;
     }
     e = launch_step(h, h->cur, true, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "step kernel");
@@ -1096,6 +1143,17 @@ int lbms_adjoint_reduce(lbms_t* h, const void* gacc, double* dL_dD)
 }
 
 long lbms_steps_done(const lbms_t* h) { return h ? h->steps : -1; }
+
+long lbms_step_launches(const lbms_t* h, long n_steps)
+{
+    if (!h) return -1;
+    if (n_steps < 1) return 0;
+    long left = n_steps - 1, launches = 1;  // the mass-writing last step
+    if (n_steps > kCallGraphMax)
+        for (int j = 0; j < 5; ++j)
+            for (; left >= kGraphLens[j]; left -= kGraphLens[j]) launches += plain_launches(h, kGraphLens[j]);
+    return launches + plain_launches(h, left);
+}
 
 const void* lbms_populations(const lbms_t* h) { return h ? h->f[h->cur] : nullptr; }
 

@@ -17,7 +17,8 @@ enum Op : int {
     OP_STEP_MASS = 1,  // the same, also writing per-block mass partials
     OP_INIT = 2,       // f+ = w_k xi from a mole-fraction chunk
     OP_MOMENTS = 3,    // xi (and J) of a cell range into a field chunk
-    OP_MASS = 4        // per-block mass partials of the current state only
+    OP_MASS = 4,       // per-block mass partials of the current state only
+    OP_FUSED = 5       // KArgs::steps stream-collide steps fin -> fout in one pass
 };
 
 // Everything a node kernel may need, dtype-agnostic; the dispatcher converts
@@ -51,6 +52,8 @@ struct KArgs {
     const uint32_t* clock_in = nullptr;  // step counter read by a step
     uint32_t* clock_out = nullptr;       // step counter written by a step
     int reverse = 0;                     // step: blocks take the grid from its end
+    int steps = 1;                       // fused pass: steps taken
+    int sms = 1;                         // multiprocessors of the device
     cudaStream_t stream = nullptr;
 };
 
@@ -72,6 +75,11 @@ cudaError_t dispatch_halo_d3q15(Op op, int dtype, const KArgs& a);
 cudaError_t dispatch_halo_d1q3(Op op, int dtype, const KArgs& a);
 cudaError_t dispatch_halo_d2q4(Op op, int dtype, const KArgs& a);
 cudaError_t dispatch_halo_d3q6(Op op, int dtype, const KArgs& a);
+
+// Most steps a fused pass takes (OP_FUSED), or 1 where the solver takes single
+// steps only: per-lattice limits (kf_*.cu) within the rule of fused_depth (lbms.cu).
+int fused_limit_of(int lattice, int n_species);
+cudaError_t dispatch_fused(int lattice, const KArgs& a);
 
 // Number of blocks a node kernel over `cells` nodes is launched with.
 inline uint32_t node_blocks(uint32_t cells) { return (cells + kBlock - 1) / kBlock; }

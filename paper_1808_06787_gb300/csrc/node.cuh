@@ -50,38 +50,42 @@
 #pragma once
 
 #include "lattice.cuh"
+#include "vec.cuh"
 
 namespace lbms {
 
-// Reciprocal used by the per-node solve: the fast hardware approximation in
-// FP32 (well inside the FP32 tolerance), the IEEE division in FP64.
-__device__ __forceinline__ float recip(float v) { return __fdividef(1.0f, v); }
-__device__ __forceinline__ double recip(double v) { return 1.0 / v; }
+// The node functions are written with the explicit operations of vec.cuh and
+// take a value type V: float and double (one node), or f2 (two nodes, FP32).
 
 // Lambda_1/2 = K^{-1} (B/2) and Lambda_2/2 (Eq. 3-16, or = Lambda_1/2 for SRT) from
 // all S+1 mole fractions and the halved inverse diffusivities invDh[i][j] =
 // 1/(2 D_ij).
-template <int S, typename T, typename InvD>
-__device__ __forceinline__ void relaxation_matrices(const T (&xi)[S + 1], const InvD& invDh,
-                                                    T cs2inv, int relax, T (&L1)[S][S],
-                                                    T (&L2)[S][S])
+template <int S, typename V, typename InvD>
+__device__ __forceinline__ void relaxation_matrices(const V (&xi)[S + 1], const InvD& invDh,
+                                                    typename Vec<V>::scalar cs2inv, int relax,
+                                                    V (&L1)[S][S], V (&L2)[S][S])
 {
-    T K[S][S];
+    using T = typename Vec<V>::scalar;
+    using A = Vec<V>;
+    const V kap = A::all(cs2inv);
+    V K[S][S];
 #pragma unroll
     for (int i = 0; i < S; ++i) {
 #pragma unroll
         for (int j = 0; j < S; ++j) {
-            T b;  // B/2
+            V b;  // B/2
             if (i != j) {
-                b = xi[i] * (invDh[i][S] - invDh[i][j]);  // Eq. 2-10, i != j
+                b = vmul(xi[i], A::all(invDh[i][S] - invDh[i][j]));  // Eq. 2-10, i != j
             } else {
-                b = xi[i] * invDh[i][S];  // Eq. 2-10, i == j
+                // Eq. 2-10, i == j: xi_i / D_in + sum_{k != i} xi_k / D_ik
+                const int k0 = i == 0 ? 1 : 0;
+                b = vfma(xi[i], A::all(invDh[i][S]), vmul(xi[k0], A::all(invDh[i][k0])));
 #pragma unroll
-                for (int k = 0; k <= S; ++k)
-                    if (k != i) b += xi[k] * invDh[i][k];
+                for (int k = k0 + 1; k <= S; ++k)
+                    if (k != i) b = vfma(xi[k], A::all(invDh[i][k]), b);
             }
             L1[i][j] = b;
-            K[i][j] = i == j ? b + cs2inv : b;
+            K[i][j] = i == j ? vadd(b, kap) : b;
         }
     }
     if constexpr (S == 2) {
@@ -90,85 +94,97 @@ __device__ __forceinline__ void relaxation_matrices(const T (&xi)[S + 1], const 
         // h = N_ii / d, Eq. 3-16 for l = 2h reads lambda_2/2 = 4 (N_ii - d) /
         // (N_ii - 4 d), so one reciprocal of d (N_00 - 4d) (N_11 - 4d) gives 1/d
         // and both diagonal entries of Lambda_2/2 (N_ii - 4d < 0 for l < 8).
-        const T d = K[0][0] * K[1][1] - K[0][1] * K[1][0];
-        const T b00 = L1[0][0], b01 = L1[0][1], b10 = L1[1][0], b11 = L1[1][1];
-        const T n00 = K[1][1] * b00 - K[0][1] * b10;
-        const T n01 = K[1][1] * b01 - K[0][1] * b11;
-        const T n10 = K[0][0] * b10 - K[1][0] * b00;
-        const T n11 = K[0][0] * b11 - K[1][0] * b01;
-        T rdet;
+        // (K_01 = b_01 and K_10 = b_10, so the product b_01 b_10 serves three times.)
+        const V b00 = L1[0][0], b01 = L1[0][1], b10 = L1[1][0], b11 = L1[1][1];
+        const V mm = vnmul(b01, b10);
+        const V d = vfma(K[0][0], K[1][1], mm);
+        const V n00 = vfma(K[1][1], b00, mm);
+        const V n01 = vfma(K[1][1], b01, vnmul(b01, b11));
+        const V n10 = vfma(K[0][0], b10, vnmul(b10, b00));
+        const V n11 = vfma(K[0][0], b11, mm);
+        V rdet;
         if (relax != LBMS_RELAX_SRT) {  // Eq. 3-16 (the frozen mode uses it too)
-            const T p0 = n00 - T(4) * d, p1 = n11 - T(4) * d;
-            const T pp = p0 * p1;
-            const T inv = recip(d * pp);
-            rdet = inv * pp;
-            const T q = inv * d;
-            L2[0][0] = T(4) * (n00 - d) * (q * p1);
-            L2[1][1] = T(4) * (n11 - d) * (q * p0);
+            const V m4 = A::all(T(-4));
+            const V p0 = vfma(m4, d, n00), p1 = vfma(m4, d, n11);
+            const V pp = vmul(p0, p1);
+            const V inv = recip(vmul(d, pp));
+            rdet = vmul(inv, pp);
+            const V q4 = vmul(A::all(T(4)), vmul(inv, d));
+            L2[0][0] = vmul(vsub(n00, d), vmul(q4, p1));
+            L2[1][1] = vmul(vsub(n11, d), vmul(q4, p0));
         } else {
             rdet = recip(d);
         }
-        L1[0][0] = n00 * rdet;
-        L1[0][1] = n01 * rdet;
-        L1[1][0] = n10 * rdet;
-        L1[1][1] = n11 * rdet;
+        L1[0][0] = vmul(n00, rdet);
+        L1[0][1] = vmul(n01, rdet);
+        L1[1][0] = vmul(n10, rdet);
+        L1[1][1] = vmul(n11, rdet);
         L2[0][1] = L1[0][1];
         L2[1][0] = L1[1][0];
         if (relax == LBMS_RELAX_SRT) {
             L2[0][0] = L1[0][0];
             L2[1][1] = L1[1][1];
         }
-        return;
     } else {
+        const V one = A::all(T(1));
 #pragma unroll
         for (int p = 0; p < S; ++p) {
-            const T inv = recip(K[p][p]);
+            const V inv = recip(K[p][p]);
 #pragma unroll
             for (int j = 0; j < S; ++j) {
-                K[p][j] *= inv;
-                L1[p][j] *= inv;
+                K[p][j] = vmul(K[p][j], inv);
+                L1[p][j] = vprod(L1[p][j], inv);
             }
 #pragma unroll
             for (int r = 0; r < S; ++r) {
                 if (r == p) continue;
-                const T fac = K[r][p];
+                const V fac = K[r][p];
 #pragma unroll
                 for (int j = 0; j < S; ++j) {
-                    K[r][j] -= fac * K[p][j];
-                    L1[r][j] -= fac * L1[p][j];
+                    if (p == 0 && j != 0 && j != r) {
+                        // the first elimination of an off-diagonal entry forms it in the same operation
+                        const V dc = A::all(invDh[r][S] - invDh[r][j]);
+                        K[r][j] = vfma(xi[r], dc, vnmul(fac, K[p][j]));
+                        L1[r][j] = vfma(xi[r], dc, vnmul(fac, L1[p][j]));
+                    } else {
+                        K[r][j] = vfma(vneg(fac), K[p][j], K[r][j]);
+                        L1[r][j] = vfma(vneg(fac), L1[p][j], L1[r][j]);
+                    }
                 }
             }
         }
-    }
 #pragma unroll
-    for (int i = 0; i < S; ++i)
+        for (int i = 0; i < S; ++i)
 #pragma unroll
-        for (int j = 0; j < S; ++j) L2[i][j] = L1[i][j];
-    if (relax != LBMS_RELAX_SRT) {  // Eq. 3-16 (the frozen mode uses it too)
-        // Eq. 3-16 with l = 2 h: lambda_2/2 = 4 (h - 1) / (h - 4)
+            for (int j = 0; j < S; ++j) L2[i][j] = L1[i][j];
+        if (relax != LBMS_RELAX_SRT) {  // Eq. 3-16 (the frozen mode uses it too)
+            // Eq. 3-16 with l = 2 h: lambda_2/2 = 4 (h - 1) / (h - 4)
+            const V four = A::all(T(4));
 #pragma unroll
-        for (int i = 0; i < S; ++i) {
-            const T h = L1[i][i];
-            L2[i][i] = T(4) * (h - T(1)) * recip(h - T(4));  // Eq. 3-16, i == j
+            for (int i = 0; i < S; ++i) {
+                const V h = L1[i][i];
+                L2[i][i] = vmul(vmul(four, vsub(h, one)), recip(vsub(h, four)));
+            }
         }
     }
 }
 
 // xi_i = sum_k f_k^i (Eq. 3-15) and xi_n = 1 - sum (Eq. 2-3b).
-template <int LAT, int S, typename T>
-__device__ __forceinline__ void mole_fractions(const T (&f)[S][Lattice<LAT>::Q], T (&xi)[S + 1])
+template <int LAT, int S, typename V>
+__device__ __forceinline__ void mole_fractions(const V (&f)[S][Lattice<LAT>::Q], V (&xi)[S + 1])
 {
+    using T = typename Vec<V>::scalar;
     constexpr int Q = Lattice<LAT>::Q;
-    T sum = T(0);
+    V sum;
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-        T x = f[s][0];
+        V x = f[s][0];
 #pragma unroll
-        for (int k = 1; k < Q; ++k) x += f[s][k];
+        for (int k = 1; k < Q; ++k) x = vadd(x, f[s][k]);
         xi[s] = x;
-        sum += x;
+        sum = s == 0 ? x : vadd(sum, x);
     }
-    xi[S] = T(1) - sum;
+    xi[S] = vsub(Vec<V>::all(T(1)), sum);
 }
 
 // Final rounding of the rest population from the exact value hi + lo.
@@ -189,78 +205,99 @@ __device__ __forceinline__ float round_rest(float hi, float lo, uint32_t h)
     // hi = RN(hi + lo) and |lo| <= half the gap to the neighbour on lo's side;
     // moving to that neighbour with probability |lo| / gap is unbiased.
     // (lo != 0 implies hi != 0; the neighbour of a finite non-zero float on the
-    // side of lo is one step of its bit pattern away from or toward zero)
+    // side of lo is one step of its bit pattern away from zero, or toward it where
+    // the signs differ; with lo = 0 the test fails)
     const float u = (float)(h >> 8) * 0x1p-24f;
-    const int step = ((lo > 0.0f) == (hi > 0.0f)) ? 1 : -1;
-    const float nb = __int_as_float(__float_as_int(hi) + step);
-    return (lo != 0.0f && fabsf(lo) > u * fabsf(nb - hi)) ? nb : hi;
+    const uint32_t same = ~(__float_as_uint(lo) ^ __float_as_uint(hi)) & 0x80000000u;  // equal signs
+    const float nb = __uint_as_float(__float_as_uint(hi) - 1u + (same >> 30));
+    return fabsf(lo) > u * fabsf(nb - hi) ? nb : hi;
 }
 
 __device__ __forceinline__ double round_rest(double hi, double, uint32_t) { return hi; }
 
 // Error-free sum a + b = s + e (Knuth's two-sum).
-template <typename T>
-__device__ __forceinline__ void two_sum(T a, T b, T& s, T& e)
+template <typename V>
+__device__ __forceinline__ void two_sum(V a, V b, V& s, V& e)
 {
-    s = a + b;
-    const T bp = s - a;
-    e = (a - (s - bp)) + (b - bp);
+    s = vadd(a, b);
+    const V bp = vsub(s, a);
+    e = vadd(vsub(a, vsub(s, bp)), vsub(b, bp));
+}
+
+// The rounding key of a node's collision: distinct per node and step, one hash
+// per node; species i draws an odd multiple of it offset by a species constant
+// (a bijection of a uniform 32-bit number, so again uniform).
+__device__ __forceinline__ uint32_t species_draw(uint32_t hn, int i)
+{
+    return (hn ^ (0x9e3779b9u * (uint32_t)(i + 1))) * 0x85ebca6bu;
+}
+
+__device__ __forceinline__ float absorb(float f0, float moved, uint32_t hn, int i)
+{
+    float h, l;
+    two_sum(f0, moved, h, l);
+    return round_rest(h, l, species_draw(hn, i));
+}
+__device__ __forceinline__ double absorb(double f0, double moved, uint32_t, int) { return vadd(f0, moved); }
+
+// The hashes of one node, or of the two nodes of a packed pair.
+struct Key2 {
+    uint32_t a, b;
+};
+__device__ __forceinline__ Key2 mix32(Key2 k) { return {mix32(k.a), mix32(k.b)}; }
+__device__ __forceinline__ f2 absorb(f2 f0, f2 moved, Key2 hn, int i)
+{
+    f2 h, l;
+    two_sum(f0, moved, h, l);
+    return pack2(round_rest(lo(h), lo(l), species_draw(hn.a, i)), round_rest(hi(h), hi(l), species_draw(hn.b, i)));
 }
 
 // In-place collision in the pair form (see the header comment) with the half
 // matrices L1h = Lambda_1/2, L2h = Lambda_2/2; `key` (distinct per node and
 // step) seeds the stochastic rounding of the rest population (FP32 only).
-template <int LAT, int S, typename T>
-__device__ __forceinline__ void collide(T (&f)[S][Lattice<LAT>::Q], const T (&xi)[S + 1],
-                                        const T (&L1h)[S][S], const T (&L2h)[S][S], uint32_t key)
+template <int LAT, int S, typename V, typename Key>
+__device__ __forceinline__ void collide(V (&f)[S][Lattice<LAT>::Q], const V (&xi)[S + 1],
+                                        const V (&L1h)[S][S], const V (&L2h)[S][S], Key key)
 {
     using L = Lattice<LAT>;
+    using T = typename Vec<V>::scalar;
     // sum of the moving populations' increments f_k - f+_k (each exact: f+_k is
     // within a factor two of f_k); its rounding is far below an ulp of f_0
-    T moved[S];
-#pragma unroll
-    for (int i = 0; i < S; ++i) moved[i] = T(0);
+    V moved[S];
 #pragma unroll
     for (int pr = 0; pr < L::NPAIR; ++pr) {
         const int ka = L::K0 + 2 * pr, kb = ka + 1;
-        const T wp2 = T(2.0 * L::w(ka));
-        T sym[S], asym[S];  // g_k + g_kbar and g_k - g_kbar
+        const V mwp2 = Vec<V>::all(T(-2.0 * L::w(ka)));
+        V sym[S], asym[S];  // g_k + g_kbar and g_k - g_kbar
 #pragma unroll
         for (int j = 0; j < S; ++j) {
-            sym[j] = (f[j][ka] + f[j][kb]) - wp2 * xi[j];
-            asym[j] = f[j][ka] - f[j][kb];
+            sym[j] = vfma(mwp2, xi[j], vadd(f[j][ka], f[j][kb]));
+            asym[j] = vsub(f[j][ka], f[j][kb]);
         }
 #pragma unroll
         for (int i = 0; i < S; ++i) {
-            T ds = T(0), da = T(0);
+            V ds = vprod(L2h[i][0], sym[0]), da = vprod(L1h[i][0], asym[0]);
 #pragma unroll
-            for (int j = 0; j < S; ++j) {
-                ds += L2h[i][j] * sym[j];
-                da += L1h[i][j] * asym[j];
+            for (int j = 1; j < S; ++j) {
+                ds = vfma(L2h[i][j], sym[j], ds);
+                da = vfma(L1h[i][j], asym[j], da);
             }
-            const T na = f[i][ka] - (ds + da);
-            const T nb = f[i][kb] - (ds - da);
-            if (ka == 0) {
-                // no rest velocity: population 0 is the absorber below
-                moved[i] += f[i][kb] - nb;
-            } else {
-                moved[i] += (f[i][ka] - na) + (f[i][kb] - nb);
+            const V na = vsub(f[i][ka], vadd(ds, da));
+            const V nb = vsub(f[i][kb], vsub(ds, da));
+            V inc = vsub(f[i][kb], nb);
+            if (ka != 0) {  // (without a rest velocity, population 0 is the absorber below)
+                inc = vadd(vsub(f[i][ka], na), inc);
                 f[i][ka] = na;
             }
+            moved[i] = pr == 0 ? inc : vadd(moved[i], inc);
             f[i][kb] = nb;
         }
     }
     // population 0 (the rest population; on lattices without one, the first
-    // moving population): f+_0 = f_0 + sum_{k != 0} (f_k - f+_k); one hash per
-    // node, and per species an odd multiple of it offset by a species constant
-    // (a bijection of a uniform 32-bit number, so again uniform)
-    const uint32_t hn = mix32(key);
+    // moving population): f+_0 = f_0 + sum_{k != 0} (f_k - f+_k)
+    const Key hn = mix32(key);
 #pragma unroll
-    for (int i = 0; i < S; ++i) {
-        T hi, lo;
-        two_sum(f[i][0], moved[i], hi, lo);
-        f[i][0] = round_rest(hi, lo, (hn ^ (0x9e3779b9u * (uint32_t)(i + 1))) * 0x85ebca6bu);
-    }
+    for (int i = 0; i < S; ++i) f[i][0] = absorb(f[i][0], moved[i], hn, i);
 }
 
 // Grid geometry shared by the node kernels.  Coordinates of a linear node

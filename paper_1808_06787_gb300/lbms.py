@@ -39,7 +39,7 @@ EXPORTED = (
     "lbms_workspace_size", "lbms_create", "lbms_set_state", "lbms_set_boundary",
     "lbms_set_reference", "lbms_step",
     "lbms_moments", "lbms_gradient",
-    "lbms_mass", "lbms_mass_noalloc", "lbms_status", "lbms_steps_done", "lbms_populations",
+    "lbms_mass", "lbms_mass_noalloc", "lbms_status", "lbms_steps_done", "lbms_step_launches", "lbms_populations",
     "lbms_last_error",
     "lbms_destroy",
     "lbms_batch_workspace_size", "lbms_batch_create", "lbms_batch_set_state", "lbms_batch_step",
@@ -107,6 +107,8 @@ def load(build_if_missing: bool = True) -> ctypes.CDLL:
         L.lbms_status.restype = I
         L.lbms_steps_done.argtypes = [P]
         L.lbms_steps_done.restype = ctypes.c_long
+        L.lbms_step_launches.argtypes = [P, ctypes.c_long]
+        L.lbms_step_launches.restype = ctypes.c_long
         L.lbms_populations.argtypes = [P]
         L.lbms_populations.restype = P
         L.lbms_last_error.argtypes = [P]
@@ -514,6 +516,10 @@ class Solver:
     @property
     def steps_done(self) -> int:
         return lbms_steps_done(self._h)
+
+    def step_launches(self, n: int) -> int:
+        """Kernel launches that ``step(n)`` makes."""
+        return int(load().lbms_step_launches(self._h, int(n)))
 
     def close(self) -> None:
         if getattr(self, "_h", None):

@@ -1,0 +1,83 @@
+"""Passes of several steps (fused.cuh) against the single steps.
+
+lbms_step takes large planes and lines several steps at a time; lbms_recompute always
+launches single steps.  Both use the same node functions and rounding keys, so the
+populations must be equal bit for bit, at every edge: strips that end inside the grid, a
+last part with fewer rows, walls and wraps on every face, step counts that leave
+remainders, and rows of odd length.
+"""
+
+import numpy as np
+import pytest
+
+import synthetic as sy
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1808_06787_gb300 as p
+
+    p.load()
+
+
+def _solver(lattice, n, grid, faces, relax, seed=5):
+    from paper_1808_06787_gb300 import Solver
+
+    kind = {"p": "periodic", "w": "noflux"}
+    s = Solver(lattice, sy.random_D(n, seed=seed), grid, bc=[kind[c] for c in faces], relax=relax)
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    x = torch.rand(s.field_shape, device="cuda", dtype=torch.float64, generator=g) + 0.05
+    s.set_state((x / x.sum(0, keepdim=True)).float())
+    return s
+
+
+CASES = [  # lattice, species, grid, faces
+    ("D2Q5", 3, (4099, 401), "wwpppp"), ("D2Q5", 3, (56, 30011), "pppppp"), ("D2Q5", 3, (1251, 1258), "wwwwpp"),
+    ("D2Q5", 3, (65537, 24), "ppwwpp"), ("D2Q5", 2, (1025, 1027), "wwwwpp"), ("D2Q4", 3, (1280, 1236), "pppppp"),
+    ("D2Q4", 2, (57, 18403), "wwwwpp"), ("D2Q9", 2, (1024, 1024), "wwwwpp"), ("D2Q9", 3, (1053, 1000), "wwwwpp"),
+    ("D2Q9", 3, (1000, 1053), "ppwwpp"), ("D2Q9", 4, (701, 751), "wwpppp"), ("D2Q9", 5, (729, 720), "wwwwpp"),
+    ("D2Q5", 5, (1111, 480), "ppwwpp"), ("D2Q5", 4, (56, 9400), "wwpppp"),
+    ("D1Q3", 3, (1,), "pppppp"), ("D1Q3", 2, (7,), "wwpppp"), ("D1Q3", 3, (112,), "wwpppp"),
+    ("D1Q3", 3, (113,), "pppppp"), ("D1Q3", 2, (127,), "pppppp"), ("D1Q3", 3, (100003,), "wwpppp"),
+]
+
+
+@pytest.mark.parametrize("relax", ["magic", "srt"])
+@pytest.mark.parametrize("lattice,n,grid,faces", CASES)
+def test_fused_passes_equal_single_steps(lattice, n, grid, faces, relax):
+    a = _solver(lattice, n, grid, faces, relax)
+    for steps in (2, 3, 4, 9, 20):
+        assert a.step_launches(steps) < steps or steps == 2, "not fused"
+        f0, t0 = a.get_state(), a.steps_done
+        out = torch.empty((steps,) + a.state_shape, device="cuda")
+        a.recompute(f0, t0, steps, out)
+        a.step(steps)
+        assert torch.equal(a.get_state(), out[-1]), steps
+        if steps == 9:  # the fluxes need the state one step back
+            J = a.moments(flux=True)[1]
+            b = _solver(lattice, n, grid, faces, relax)
+            b.set_state_raw(out[-2].contiguous(), t0 + steps - 1)
+            b.step(1)
+            assert torch.equal(b.moments(flux=True)[1], J)
+    # a long call goes through the captured pieces of 32 .. 2 steps
+    f0, t0 = a.get_state(), a.steps_done
+    a.step(71)
+    out = torch.empty((71,) + a.state_shape, device="cuda") if np.prod(a.state_shape) < 1 << 22 else None
+    if out is not None:
+        a.recompute(f0, t0, 71, out)
+        assert torch.equal(a.get_state(), out[-1])
+    assert a.steps_done == t0 + 71
+
+
+def test_launch_counts():
+    a = _solver("D2Q5", 3, (40, 40), "pppppp", "magic")  # a small plane takes single steps
+    assert [a.step_launches(n) for n in (0, 1, 2, 20, 71)] == [0, 1, 2, 20, 71]
+    b = _solver("D1Q3", 3, (500,), "pppppp", "magic")  # eight at a time, the last by itself
+    assert [b.step_launches(n) for n in (1, 2, 9, 10, 20)] == [1, 2, 2, 3, 4]
+    assert b.step_launches(71) == 1 + 2 * 4 + 1 + 1
