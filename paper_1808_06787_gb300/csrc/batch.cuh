@@ -249,15 +249,9 @@ __global__ void __launch_bounds__(kBlock) k_batch_init(BatchParams<T> p)
     if (local >= d.g.cells) return;
     const T* src = p.x_in + p.field_off[id];
     T xi[S + 1];
-    double sum = 0.0;
-    bool finite = true;
 #pragma unroll
-    for (int s = 0; s <= S; ++s) {
-        xi[s] = src[(size_t)s * d.g.cells + local];
-        sum += (double)xi[s];
-        finite &= (bool)isfinite((double)xi[s]);
-    }
-    if (!finite || !(fabs(sum - 1.0) <= 1e-5)) atomicOr(p.status, LBMS_FLAG_INIT);
+    for (int s = 0; s <= S; ++s) xi[s] = src[(size_t)s * d.g.cells + local];
+    if (!initial_ok<S, T>(xi)) atomicOr(p.status, LBMS_FLAG_INIT);
     const uint32_t cell = d.base + local;
 #pragma unroll
     for (int s = 0; s < S; ++s) {

