@@ -62,7 +62,7 @@ int lattice_dim(int lat)
 struct BLayout {
     uint32_t total_blocks = 0, total_nodes = 0;
     size_t f_bytes = 0, off_f1 = 0, off_partials = 0, off_mass = 0, off_inst = 0, off_blk = 0,
-           off_invD = 0, off_clock = 0, off_foff = 0, off_xb = 0, off_status = 0, off_staging = 0,
+           off_invD = 0, off_clock = 0, off_foff = 0, off_xb = 0, off_fixed = 0, off_status = 0, off_staging = 0,
            staging_bytes = 0, total = 0;
 };
 
@@ -98,7 +98,8 @@ bool batch_layout(int lat, int n, int count, const int* grids, int dtype, BLayou
     L->off_foff = L->off_clock + align_up((size_t)count * 2 * sizeof(uint32_t));
     L->off_xb = L->off_foff + align_up((size_t)count * sizeof(long long));
     // Dirichlet compositions [count][6][S]
-    L->off_status = L->off_xb + align_up((size_t)count * 6 * (n - 1) * es);
+    L->off_fixed = L->off_xb + align_up((size_t)count * 6 * (n - 1) * es);
+    L->off_status = L->off_fixed + (dtype == LBMS_F64 ? align_up((size_t)count * sizeof(FixedTable)) : 0);
     L->off_staging = L->off_status + kAlign;
     // staging: large enough for the biggest instance's fields, at most 16 MiB beyond that
     const size_t biggest = (size_t)max_field * n * (1 + dim) * es;
@@ -160,6 +161,7 @@ struct lbms_batch_s {
     BatchInst* inst_dev = nullptr;
     uint32_t* blk_dev = nullptr;
     void* invD_dev = nullptr;
+    FixedTable* fixed_dev = nullptr;      // [count] coefficients of the fixed-point collision (FP64)
     uint32_t* clock = nullptr;
     long long* foff_dev = nullptr;
     void* xb_dev = nullptr;               // [count][6][S] Dirichlet compositions, solver dtype
@@ -219,6 +221,7 @@ BArgs bargs(const lbms_batch_t* b, cudaStream_t st, uint32_t b0, uint32_t b1)
     a.blk_inst = b->blk_dev;
     a.inst = b->inst_dev;
     a.invD = b->invD_dev;
+    a.fixed = b->fixed_dev;
     a.n_species = b->n;
     a.relax = b->relax;
     a.clock = b->clock;
@@ -418,6 +421,7 @@ int lbms_batch_create(lbms_batch_t** out, int lattice, int n_species, int count,
     b->clock = reinterpret_cast<uint32_t*>(b->ws + L.off_clock);
     b->foff_dev = reinterpret_cast<long long*>(b->ws + L.off_foff);
     b->xb_dev = b->ws + L.off_xb;
+    b->fixed_dev = reinterpret_cast<FixedTable*>(b->ws + L.off_fixed);
     b->dirichlet.assign(count, 0u);
     b->xb_set.assign(count, 0u);
     b->status = reinterpret_cast<uint32_t*>(b->ws + L.off_status);
@@ -429,6 +433,7 @@ int lbms_batch_create(lbms_batch_t** out, int lattice, int n_species, int count,
     b->packed_off.resize(count);
     std::vector<uint32_t> blk(L.total_blocks);
     std::vector<char> invD((size_t)count * n * n * b->es);
+    std::vector<FixedTable> fixed(dtype == LBMS_F64 ? count : 0);
     uint32_t block = 0;
     long long off = 0;
     for (int c = 0; c < count; ++c) {
@@ -459,6 +464,12 @@ int lbms_batch_create(lbms_batch_t** out, int lattice, int n_species, int count,
         off += (long long)n * ka.cells;
         if (ka.cells > maxcells) maxcells = ka.cells;
         const double* Dc = D + (size_t)c * n * n;
+        if (dtype == LBMS_F64) {
+            double full[LBMS_MAX_SPECIES][LBMS_MAX_SPECIES] = {};
+            for (int i = 0; i < n; ++i)
+                for (int j = 0; j < n; ++j) full[i][j] = i == j ? 0.0 : 1.0 / Dc[i * n + j];
+            fixed[c] = fixed_table(n, full, lattice_cs2(lattice), relax);
+        }
         for (int i = 0; i < n; ++i)
             for (int j = 0; j < n; ++j) {
                 // halved inverse diffusivities (relaxation_matrices takes 1/(2 D_ij))
@@ -484,6 +495,9 @@ int lbms_batch_create(lbms_batch_t** out, int lattice, int n_species, int count,
                             b->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b->invD_dev, invD.data(), invD.size(), cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess && dtype == LBMS_F64)
+        e = cudaMemcpyAsync(b->fixed_dev, fixed.data(), fixed.size() * sizeof(FixedTable), cudaMemcpyHostToDevice,
+                            b->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->status, 0, sizeof(uint32_t), b->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->clock, 0, sizeof(uint32_t) * 2 * count, b->stream);
     // the host tables are copied from pageable memory: wait before they go

@@ -33,6 +33,7 @@ struct BArgs {
     const uint32_t* blk_inst = nullptr;       // [total_blocks] instance of each block
     const BatchInst* inst = nullptr;          // [count]
     const void* invD = nullptr;               // [count][n][n] 1/(2 D_ij), element type
+    const FixedTable* fixed = nullptr;        // [count] coefficients of the fixed-point collision (FP64)
     int n_species = 2;
     int relax = LBMS_RELAX_MAGIC;
     uint32_t* clock = nullptr;                // [count][2] step counters
@@ -67,6 +68,7 @@ struct BatchParams {
     const uint32_t* __restrict__ blk_inst;
     const BatchInst* __restrict__ inst;
     const T* __restrict__ invD;
+    const FixedTable* __restrict__ fixed;
     int relax;
     uint32_t* clock;
     int parity;
@@ -106,12 +108,17 @@ __global__ void __launch_bounds__(kBlock) k_batch_step(BatchParams<T> p, const T
         const uint32_t cell = d.base + local;
         T f[S][Q];
         pull<LAT, S, T>(p.fin, plane, cell, h, f, DIR ? xb + (size_t)id * 6 * S : static_cast<const T*>(nullptr));
-        mole_fractions<LAT, S, T>(f, xi);
+        bool done = false;
+        if constexpr (sizeof(T) == 4 || MASS) mole_fractions<LAT, S, T>(f, xi);
         if (MASS) check_range<S, T>(xi, p.status);  // once per step call
-        const InvDView<T> iv{p.invD + (size_t)id * (S + 1) * (S + 1), S + 1};
-        T L1[S][S], L2[S][S];
-        relaxation_matrices<S, T>(xi, iv, T(1.0 / L::cs2()), p.relax, L1, L2);
-        collide<LAT, S, T>(f, xi, L1, L2, mix32(step * 0x9e3779b9u) ^ (local * 0x27d4eb2du));
+        if constexpr (sizeof(T) == 8) done = try_fixed<LAT, S>(f, p.fixed[id]);
+        if (!done) {
+            if constexpr (sizeof(T) == 8 && !MASS) mole_fractions<LAT, S, T>(f, xi);
+            const InvDView<T> iv{p.invD + (size_t)id * (S + 1) * (S + 1), S + 1};
+            T L1[S][S], L2[S][S];
+            relaxation_matrices<S, T>(xi, iv, T(1.0 / L::cs2()), p.relax, L1, L2);
+            collide<LAT, S, T>(f, xi, L1, L2, mix32(step * 0x9e3779b9u) ^ (local * 0x27d4eb2du));
+        }
 #pragma unroll
         for (int s = 0; s < S; ++s)
 #pragma unroll
@@ -330,6 +337,7 @@ cudaError_t batch_launch(BatchOp op, const BArgs& a)
     p.blk_inst = a.blk_inst;
     p.inst = a.inst;
     p.invD = static_cast<const T*>(a.invD);
+    p.fixed = a.fixed;
     p.relax = a.relax;
     p.clock = a.clock;
     p.parity = a.parity;

@@ -6,9 +6,34 @@
 
 #include <math.h>
 
+#include "fixed.cuh"
 #include "node.cuh"
 
 namespace lbms {
+
+// The fixed-point collision's coefficients, an argument of the FP64 kernels only.
+template <typename T>
+struct FixedArg {};
+template <>
+struct FixedArg<double> {
+    FixedTable table;
+};
+
+// Collision of one FP64 node in fixed point (fixed.cuh), for binary and ternary mixtures;
+// false where the FP64 arithmetic has to take it.
+template <int LAT, int S>
+__device__ __forceinline__ bool try_fixed(double (&f)[S][Lattice<LAT>::Q], const FixedTable& t)
+{
+    if constexpr (S <= 2) {
+        if (t.on) return collide_fixed<Lattice<LAT>, S>(f, t);
+    }
+    return false;
+}
+template <int LAT, int S, typename Any>
+__device__ __forceinline__ bool try_fixed(float (&)[S][Lattice<LAT>::Q], const Any&)
+{
+    return false;
+}
 
 template <typename T>
 struct Coeffs {
@@ -49,6 +74,7 @@ struct StepParams {
     uint32_t* clock_out;
     const T* __restrict__ xb;  // Dirichlet face compositions [6][S]
     Halo<T> halo;              // slab cuts: receive buffers of fin's parity, send buffers
+    FixedArg<T> fixed;
     int reverse;               // blocks take the grid from its end (block b does block n - 1 - b)
     Coeffs<T> co;
 };
@@ -205,12 +231,80 @@ __device__ __forceinline__ void write_mass_partials(const float (&xi)[S + 1], bo
     block_fixed_partials<S + 1>(q, static_cast<long long*>(m.partials) + (size_t)row * (S + 1));
 }
 
+// A 128-bit integer, for the exact sums of FP64 mole fractions in units of 2^-118.
+struct Wide {
+    uint64_t hi, lo;
+};
+__device__ __forceinline__ Wide add(Wide a, Wide b)
+{
+    Wide r;
+    r.lo = a.lo + b.lo;
+    r.hi = a.hi + b.hi + (r.lo < a.lo ? 1 : 0);
+    return r;
+}
+__device__ __forceinline__ Wide to_wide(double v)  // zero, or 2^-65 <= |v| < 2: exact
+{
+    const uint64_t b = (uint64_t)__double_as_longlong(v);
+    const int e = (int)(b >> 52) & 0x7ff;
+    const uint64_t m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 11;  // leading bit at bit 127
+    int r = 1032 - e;
+    Wide w;
+    if (r < 64) {
+        w.hi = m >> r;
+        w.lo = m << (64 - r);
+    } else {
+        r -= 64;
+        w.hi = 0;
+        w.lo = r < 64 ? m >> r : 0;  // zero among them
+    }
+    if (b >> 63) {
+        w.lo = 0 - w.lo;
+        w.hi = ~w.hi + (w.lo == 0 ? 1 : 0);
+    }
+    return w;
+}
+
+// The mole fractions of a block as two-sum pairs.  Two-sum reductions issue some 60 FP64
+// instructions per species and warp at the FP64 rate (D3Q7 101 x 96 x 67: 178 us of the
+// mass-writing step's 366); sums of 128-bit integers are exact and take the integer pipes.
+// Blocks with a value that is not exact in those units (below 2^-65, two or more, infinite
+// or NaN) add two-sum pairs.
 template <int S>
 __device__ __forceinline__ void write_mass_partials(const double (&xi)[S + 1], bool active,
                                                     const MassOut& m, uint32_t row)
 {
     __shared__ double2 red[kBlock / 32];
+    __shared__ Wide sums[kBlock / 32][S + 1];
     double2* out = static_cast<double2*>(m.partials);
+    bool fits = true;  // zero, or from 2^-65 (the last bit is 2^-117) to below two
+#pragma unroll
+    for (int s = 0; s <= S; ++s) {
+        const uint32_t e = (uint32_t)(__double_as_longlong(xi[s]) >> 52) & 0x7ffu;
+        fits &= !active || xi[s] == 0.0 || (e >= 958u && e <= 1023u);
+    }
+    if (__syncthreads_and(fits)) {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+        for (int s = 0; s <= S; ++s) {
+            Wide w = to_wide(active ? xi[s] : 0.0);
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1)
+                w = add(w, Wide{__shfl_down_sync(0xffffffffu, w.hi, off), __shfl_down_sync(0xffffffffu, w.lo, off)});
+            if (lane == 0) sums[warp][s] = w;
+        }
+        __syncthreads();
+        if (threadIdx.x <= S) {
+            Wide w = sums[0][threadIdx.x];
+            for (int v = 1; v < (int)(blockDim.x >> 5); ++v) w = add(w, sums[v][threadIdx.x]);
+            // the four 32-bit digits, from the largest, added as a two-sum pair
+            double sum = (double)(int32_t)(w.hi >> 32) * 0x1p-22, comp = 0.0;
+            two_sum_add(sum, comp, (double)(uint32_t)w.hi * 0x1p-54);
+            two_sum_add(sum, comp, (double)(uint32_t)(w.lo >> 32) * 0x1p-86);
+            comp += (double)(uint32_t)w.lo * 0x1p-118;
+            out[(size_t)row * (S + 1) + threadIdx.x] = make_double2(sum, comp);
+        }
+        return;
+    }
 #pragma unroll
     for (int s = 0; s <= S; ++s) {
         double sum = active ? xi[s] : 0.0, comp = 0.0;
@@ -239,12 +333,14 @@ __device__ __forceinline__ uint32_t grid_block(int reverse)
 
 // Blocks per SM the FP32 step kernels are compiled for (register budget): one
 // node per thread keeps S * Q populations and the S x S matrices in registers,
-// and enough resident warps must remain to cover HBM latency.
+// and enough resident warps must remain to cover HBM latency.  FP64 binary and ternary
+// steps (fixed.cuh) at 3 blocks: D2Q5 1024^2 66.4 / 66.4 / 55 us per step at 1 / 2 / 3, D3Q7
+// 101 x 96 x 67 50.7 / 50.7 / 46 (four alike, but D2Q9 300^2 12.6 -> 15.9).
 template <int LAT, int S, typename T>
 struct StepOccupancy {
     static constexpr int P = S * Lattice<LAT>::Q;  // populations held per thread
     static constexpr int value =
-        sizeof(T) != 4 ? 1
+        sizeof(T) != 4 ? (S <= 2 ? 3 : 1)
         : Lattice<LAT>::Q <= 9 ? (S <= 2 ? 6 : (S == 3 ? 4 : (S == 4 ? 3 : 2)))
                                : (P <= 15 ? 4 : (P <= 30 ? 3 : 2));
 };
@@ -270,16 +366,21 @@ __global__ void __launch_bounds__(kBlock, StepOccupancy<LAT, S, T>::value) k_ste
         const Neighbourhood h = neighbourhood<Lattice<LAT>::DIM, HALO>(p.g, cell);
         T f[S][Q];
         pull<LAT, S, T>(p.fin, p.g, cell, h, f, p.xb, HALO ? &p.halo : nullptr);
-        mole_fractions<LAT, S, T>(f, xi);
+        bool done = false;
+        if constexpr (sizeof(T) == 4 || MASS) mole_fractions<LAT, S, T>(f, xi);
         if (MASS) check_range<S, T>(xi, p.status);  // once per lbms_step call
-        T L1[S][S], L2[S][S];
-        T xl[S + 1];
-        lambda_composition<S, T>(xi, p.co, p.relax, xl);
-        relaxation_matrices<S, T>(xl, p.co.invD, T(1.0 / L::cs2()), p.relax, L1, L2);
-        // the rounding key uses the node's index in the undivided grid, so that
-        // the slabs of a decomposed grid round as the whole grid does
-        collide<LAT, S, T>(f, xi, L1, L2,
-                           mix32(step * 0x9e3779b9u) ^ ((HALO ? cell + p.g.origin : cell) * 0x27d4eb2du));
+        if constexpr (sizeof(T) == 8) done = try_fixed<LAT, S>(f, p.fixed.table);
+        if (!done) {
+            if constexpr (sizeof(T) == 8 && !MASS) mole_fractions<LAT, S, T>(f, xi);
+            T L1[S][S], L2[S][S];
+            T xl[S + 1];
+            lambda_composition<S, T>(xi, p.co, p.relax, xl);
+            relaxation_matrices<S, T>(xl, p.co.invD, T(1.0 / L::cs2()), p.relax, L1, L2);
+            // the rounding key uses the node's index in the undivided grid, so that
+            // the slabs of a decomposed grid round as the whole grid does
+            collide<LAT, S, T>(f, xi, L1, L2,
+                               mix32(step * 0x9e3779b9u) ^ ((HALO ? cell + p.g.origin : cell) * 0x27d4eb2du));
+        }
 #pragma unroll
         for (int s = 0; s < S; ++s)
 #pragma unroll
@@ -680,6 +781,7 @@ cudaError_t launch(Op op, const KArgs& a)
         p.clock_out = a.clock_out;
         p.xb = static_cast<const T*>(a.xb);
         p.halo = make_halo<T>(a);
+        if constexpr (sizeof(T) == 8) p.fixed.table = a.fixed;
         // alternate steps take the grid from its end (undivided grids; measured
         // on one box against forward-only steps: D3Q7 256^3 +0.8 %, D3Q6 +0.5 to
         // 1.5 %, D2Q9 N = 5 +0.9 %, D2Q5 and D1Q3 +0.3 %, D3Q15 -0.2 %)

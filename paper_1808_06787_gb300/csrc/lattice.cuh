@@ -131,6 +131,21 @@ struct Lattice<LBMS_D3Q6> {
     __host__ __device__ static constexpr double cs2() { return 1.0 / 3.0; }
 };
 
+// c_s^2 of a lattice by its number (0 for none).
+inline double lattice_cs2(int lat)
+{
+    switch (lat) {
+        case LBMS_D2Q5: return Lattice<LBMS_D2Q5>::cs2();
+        case LBMS_D2Q9: return Lattice<LBMS_D2Q9>::cs2();
+        case LBMS_D3Q7: return Lattice<LBMS_D3Q7>::cs2();
+        case LBMS_D3Q15: return Lattice<LBMS_D3Q15>::cs2();
+        case LBMS_D1Q3: return Lattice<LBMS_D1Q3>::cs2();
+        case LBMS_D2Q4: return Lattice<LBMS_D2Q4>::cs2();
+        case LBMS_D3Q6: return Lattice<LBMS_D3Q6>::cs2();
+        default: return 0.0;
+    }
+}
+
 // Slab decomposition: a grid is split along its slowest axis (z for the 3D
 // lattices, y for the 2D ones, x for D1Q3), so that one layer of nodes is a
 // contiguous run of `plane` node indices.  split_c(k) is the velocity component

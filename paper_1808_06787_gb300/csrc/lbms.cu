@@ -232,6 +232,7 @@ struct lbms_s {
     size_t es = 4;
     double invD[LBMS_MAX_SPECIES][LBMS_MAX_SPECIES] = {};
     double xref[LBMS_MAX_SPECIES] = {};  // reference composition (frozen mode)
+    FixedTable fixed = {};               // FP64: coefficients of the fixed-point collision
     bool xref_set = false;
     char* ws = nullptr;
     Layout lay{};
@@ -323,6 +324,7 @@ KArgs base_args(const lbms_t* h, cudaStream_t st)
     a.n_species = h->n;
     memcpy(a.invD, h->invD, sizeof(a.invD));
     memcpy(a.xref, h->xref, sizeof(a.xref));
+    a.fixed = h->fixed;
     a.status = h->status;
     a.fixed_shift = h->fixed_shift;
     a.sms = h->sms;
@@ -638,6 +640,7 @@ int lbms_create(lbms_t** out, int lattice, int n_species, const int grid[3], con
     h->depth = fused_depth(h);
     for (int i = 0; i < n; ++i)
         for (int j = 0; j < n; ++j) h->invD[i][j] = i == j ? 0.0 : 1.0 / D[i * n + j];
+    if (dtype == LBMS_F64) h->fixed = fixed_table(n, h->invD, lattice_cs2(lattice), relax);
     h->ws = static_cast<char*>(workspace);
     h->lay = L;
     h->f[0] = h->ws + L.off_f0;

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "fixed.cuh"
 #include "lbms.h"
 
 namespace lbms {
@@ -46,6 +47,7 @@ struct KArgs {
     int n_species = 2;
     double invD[LBMS_MAX_SPECIES][LBMS_MAX_SPECIES] = {};  // 1 / D_ij
     double xref[LBMS_MAX_SPECIES] = {};                    // reference composition (frozen mode)
+    FixedTable fixed = {};     // FP64 solvers: the fixed-point collision's coefficients
     void* partials = nullptr;  // [blocks][n]: int64 fixed point (FP32) or double2 (FP64)
     int fixed_shift = 32;      // fraction bits of the FP32 fixed-point mass partials
     uint32_t* status = nullptr;
