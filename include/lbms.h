@@ -346,7 +346,8 @@ int lbms_adjoint_reduce(lbms_t* h, const void* gacc, double* dL_dD);
 long lbms_steps_done(const lbms_t* h);
 
 /* Kernel launches that lbms_step(h, n_steps) makes (or replays): grids beyond the
- * L2 cache take several steps per launch on the 1D and 2D lattices in F32.  0 for
+ * L2 cache take several steps per launch on the 1D and 2D lattices in F32, and so do
+ * grids too small to fill the chip.  0 for
  * n_steps < 1, -1 for a NULL handle. */
 long lbms_step_launches(const lbms_t* h, long n_steps);
 

@@ -97,8 +97,8 @@ __device__ __forceinline__ void await_previous_grid()
 // dependency on the kernel before it in the stream is relaxed, and the kernel
 // must call await_previous_grid before touching memory that grid writes or reads.
 template <typename... Params, typename... Args>
-cudaError_t launch_chained(void (*kernel)(Params...), uint32_t blocks, uint32_t threads,
-                           cudaStream_t stream, Args... args)
+cudaError_t launch_chained_shared(void (*kernel)(Params...), uint32_t blocks, uint32_t threads, size_t shared_bytes,
+                                  cudaStream_t stream, Args... args)
 {
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -106,12 +106,18 @@ cudaError_t launch_chained(void (*kernel)(Params...), uint32_t blocks, uint32_t 
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks);
     cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = shared_bytes;
     cfg.stream = stream;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, kernel, args...);
     return cudaGetLastError();
+}
+template <typename... Params, typename... Args>
+cudaError_t launch_chained(void (*kernel)(Params...), uint32_t blocks, uint32_t threads,
+                           cudaStream_t stream, Args... args)
+{
+    return launch_chained_shared(kernel, blocks, threads, 0, stream, args...);
 }
 
 // Raise the status flags for mole fractions that are non-finite or far
@@ -762,6 +768,27 @@ inline Geom make_geom(const KArgs& a)
     return g;
 }
 
+template <typename T>
+StepParams<T> make_step_params(const KArgs& a)
+{
+    StepParams<T> p;
+    p.fin = static_cast<const T*>(a.fin);
+    p.fout = static_cast<T*>(a.fout);
+    p.g = make_geom(a);
+    p.relax = a.relax;
+    p.mass.partials = a.partials;
+    p.mass.shift = a.fixed_shift;
+    p.status = a.status;
+    p.clock_in = a.clock_in;
+    p.clock_out = a.clock_out;
+    p.xb = static_cast<const T*>(a.xb);
+    p.halo = make_halo<T>(a);
+    if constexpr (sizeof(T) == 8) p.fixed.table = a.fixed;
+    p.reverse = 0;
+    p.co = make_coeffs<T>(a, 0.5);
+    return p;
+}
+
 // HALO_STEPS selects the step kernels of slabs (grids with cut faces): the
 // per-lattice translation units k_*.cu instantiate the others and kh_*.cu these,
 // so that the two halves compile in parallel.
@@ -769,24 +796,11 @@ template <int LAT, int S, typename T, bool HALO_STEPS>
 cudaError_t launch(Op op, const KArgs& a)
 {
     if (op == OP_STEP || op == OP_STEP_MASS || op == OP_MASS) {
-        StepParams<T> p;
-        p.fin = static_cast<const T*>(a.fin);
-        p.fout = static_cast<T*>(a.fout);
-        p.g = make_geom(a);
-        p.relax = a.relax;
-        p.mass.partials = a.partials;
-        p.mass.shift = a.fixed_shift;
-        p.status = a.status;
-        p.clock_in = a.clock_in;
-        p.clock_out = a.clock_out;
-        p.xb = static_cast<const T*>(a.xb);
-        p.halo = make_halo<T>(a);
-        if constexpr (sizeof(T) == 8) p.fixed.table = a.fixed;
+        StepParams<T> p = make_step_params<T>(a);
         // alternate steps take the grid from its end (undivided grids; measured
         // on one box against forward-only steps: D3Q7 256^3 +0.8 %, D3Q6 +0.5 to
         // 1.5 %, D2Q9 N = 5 +0.9 %, D2Q5 and D1Q3 +0.3 %, D3Q15 -0.2 %)
         p.reverse = HALO_STEPS ? 0 : a.reverse;
-        p.co = make_coeffs<T>(a, 0.5);
         const uint32_t tb = a.step_block;
         const uint32_t blocks = (a.cells + tb - 1) / tb;
         if constexpr (HALO_STEPS) {

@@ -22,6 +22,15 @@ enum Op : int {
     OP_FUSED = 5       // KArgs::steps stream-collide steps fin -> fout in one pass
 };
 
+// A pass of several steps over tiles of a small grid (tile.cuh).
+struct Tiles {
+    int depth;           // steps of the pass, K
+    int tx, ty, tz;      // nodes of a tile
+    int rx, ry, rz;      // nodes of its region: the tile and its margins
+    int nx, ny;          // tiles along x and y
+};
+constexpr int kTileThreads = 512;  // most nodes of a region
+
 // Everything a node kernel may need, dtype-agnostic; the dispatcher converts
 // the coefficients to the kernel's type.
 struct KArgs {
@@ -55,6 +64,7 @@ struct KArgs {
     uint32_t* clock_out = nullptr;       // step counter written by a step
     int reverse = 0;                     // step: blocks take the grid from its end
     int steps = 1;                       // fused pass: steps taken
+    Tiles tiles = {};                    // tiled pass
     int sms = 1;                         // multiprocessors of the device
     cudaStream_t stream = nullptr;
 };
@@ -82,6 +92,16 @@ cudaError_t dispatch_halo_d3q6(Op op, int dtype, const KArgs& a);
 // steps only: per-lattice limits (kf_*.cu) within the rule of fused_depth (lbms.cu).
 int fused_limit_of(int lattice, int n_species);
 cudaError_t dispatch_fused(int lattice, const KArgs& a);
+// A tiled pass of a.tiles.depth steps (kt_*.cu): two to four species, not D3Q15.
+cudaError_t dispatch_tile(int lattice, int dtype, const KArgs& a);
+template <int LAT>
+cudaError_t dispatch_tile_lattice(int dtype, const KArgs& a);
+template <> cudaError_t dispatch_tile_lattice<LBMS_D1Q3>(int dtype, const KArgs& a);
+template <> cudaError_t dispatch_tile_lattice<LBMS_D2Q4>(int dtype, const KArgs& a);
+template <> cudaError_t dispatch_tile_lattice<LBMS_D2Q5>(int dtype, const KArgs& a);
+template <> cudaError_t dispatch_tile_lattice<LBMS_D2Q9>(int dtype, const KArgs& a);
+template <> cudaError_t dispatch_tile_lattice<LBMS_D3Q6>(int dtype, const KArgs& a);
+template <> cudaError_t dispatch_tile_lattice<LBMS_D3Q7>(int dtype, const KArgs& a);
 
 // Number of blocks a node kernel over `cells` nodes is launched with.
 inline uint32_t node_blocks(uint32_t cells) { return (cells + kBlock - 1) / kBlock; }

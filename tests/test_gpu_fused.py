@@ -1,6 +1,6 @@
-"""Passes of several steps (fused.cuh) against the single steps.
+"""Passes of several steps (fused.cuh, tile.cuh) against the single steps.
 
-lbms_step takes large planes and lines several steps at a time; lbms_recompute always
+lbms_step takes large planes, lines and small grids several steps at a time; lbms_recompute always
 launches single steps.  Both use the same node functions and rounding keys, so the
 populations must be equal bit for bit, at every edge: strips that end inside the grid, a
 last part with fewer rows, walls and wraps on every face, step counts that leave
@@ -26,14 +26,16 @@ def _cuda():
     p.load()
 
 
-def _solver(lattice, n, grid, faces, relax, seed=5):
+def _solver(lattice, n, grid, faces, relax, seed=5, dtype=torch.float32):
     from paper_1808_06787_gb300 import Solver
 
-    kind = {"p": "periodic", "w": "noflux"}
-    s = Solver(lattice, sy.random_D(n, seed=seed), grid, bc=[kind[c] for c in faces], relax=relax)
+    kind = {"p": "periodic", "w": "noflux", "d": "dirichlet"}
+    held = {f: np.full(n, 1.0 / n) + np.linspace(-0.1, 0.1, n) * (1 - 2 * (f % 2)) for f in range(6) if faces[f] == "d"}
+    s = Solver(lattice, sy.random_D(n, seed=seed), grid, bc=[kind[c] for c in faces], relax=relax, dtype=dtype,
+               boundary=held, reference=np.full(n, 1.0 / n) if relax == "frozen" else None)
     g = torch.Generator(device="cuda").manual_seed(seed)
     x = torch.rand(s.field_shape, device="cuda", dtype=torch.float64, generator=g) + 0.05
-    s.set_state((x / x.sum(0, keepdim=True)).float())
+    s.set_state((x / x.sum(0, keepdim=True)).to(dtype))
     return s
 
 
@@ -45,30 +47,51 @@ CASES = [  # lattice, species, grid, faces
     ("D2Q5", 5, (1111, 480), "ppwwpp"), ("D2Q5", 4, (56, 9400), "wwpppp"),
     ("D1Q3", 3, (1,), "pppppp"), ("D1Q3", 2, (7,), "wwpppp"), ("D1Q3", 3, (112,), "wwpppp"),
     ("D1Q3", 3, (113,), "pppppp"), ("D1Q3", 2, (127,), "pppppp"), ("D1Q3", 3, (100003,), "wwpppp"),
+    ("D1Q3", 3, (8193,), "pppppp"), ("D1Q3", 2, (8300,), "wwpppp"),
 ]
+TILED = [  # small grids: tiles, margins that wrap around, walls, Dirichlet faces, both dtypes
+    ("D1Q3", 4, (8192,), "wwpppp", "f32"), ("D1Q3", 3, (5,), "pppppp", "f64"), ("D1Q3", 2, (333,), "ddpppp", "f64"),
+    ("D2Q5", 3, (1, 1), "pppppp", "f32"), ("D2Q5", 3, (3, 2), "wwpppp", "f32"), ("D2Q5", 3, (48, 40), "wwwwpp", "f32"),
+    ("D2Q5", 2, (65, 63), "ddwwpp", "f32"), ("D2Q5", 4, (129, 127), "ppddpp", "f32"), ("D2Q9", 3, (7, 100), "wwwwpp", "f32"),
+    ("D2Q9", 2, (256, 255), "pppppp", "f32"), ("D2Q9", 4, (200, 150), "wwddpp", "f32"), ("D2Q4", 3, (250, 260), "wwpppp", "f32"),
+    ("D2Q5", 3, (255, 257), "ppwwpp", "f32"), ("D2Q5", 2, (240, 40), "ddpppp", "f64"), ("D2Q5", 2, (141, 143), "wwwwpp", "f64"),
+    ("D2Q5", 3, (64, 64), "ddddpp", "f64"), ("D2Q9", 3, (79, 81), "wwwwpp", "f64"), ("D2Q4", 3, (13, 9), "pppppp", "f64"),
+    ("D3Q7", 3, (18, 17, 16), "wwwwww", "f32"), ("D3Q6", 2, (5, 3, 2), "pppppp", "f32"), ("D3Q7", 2, (25, 22, 21), "ddwwpp", "f32"),
+]
+
+
+@pytest.mark.parametrize("relax", ["magic", "srt", "frozen"])
+@pytest.mark.parametrize("lattice,n,grid,faces,dtype", TILED)
+def test_tiled_passes_equal_single_steps(lattice, n, grid, faces, dtype, relax):
+    """Grids that leave most of the chip idle take tiles with margins, several steps a pass."""
+    _compare(lattice, n, grid, faces, relax, {"f32": torch.float32, "f64": torch.float64}[dtype])
 
 
 @pytest.mark.parametrize("relax", ["magic", "srt"])
 @pytest.mark.parametrize("lattice,n,grid,faces", CASES)
 def test_fused_passes_equal_single_steps(lattice, n, grid, faces, relax):
-    a = _solver(lattice, n, grid, faces, relax)
+    _compare(lattice, n, grid, faces, relax, torch.float32)
+
+
+def _compare(lattice, n, grid, faces, relax, dtype):
+    a = _solver(lattice, n, grid, faces, relax, dtype=dtype)
     for steps in (2, 3, 4, 9, 20):
         assert a.step_launches(steps) < steps or steps == 2, "not fused"
         f0, t0 = a.get_state(), a.steps_done
-        out = torch.empty((steps,) + a.state_shape, device="cuda")
+        out = torch.empty((steps,) + a.state_shape, device="cuda", dtype=dtype)
         a.recompute(f0, t0, steps, out)
         a.step(steps)
         assert torch.equal(a.get_state(), out[-1]), steps
         if steps == 9:  # the fluxes need the state one step back
             J = a.moments(flux=True)[1]
-            b = _solver(lattice, n, grid, faces, relax)
+            b = _solver(lattice, n, grid, faces, relax, dtype=dtype)
             b.set_state_raw(out[-2].contiguous(), t0 + steps - 1)
             b.step(1)
             assert torch.equal(b.moments(flux=True)[1], J)
     # a long call goes through the captured pieces of 32 .. 2 steps
     f0, t0 = a.get_state(), a.steps_done
     a.step(71)
-    out = torch.empty((71,) + a.state_shape, device="cuda") if np.prod(a.state_shape) < 1 << 22 else None
+    out = torch.empty((71,) + a.state_shape, device="cuda", dtype=dtype) if np.prod(a.state_shape) < 1 << 22 else None
     if out is not None:
         a.recompute(f0, t0, 71, out)
         assert torch.equal(a.get_state(), out[-1])
@@ -76,8 +99,8 @@ def test_fused_passes_equal_single_steps(lattice, n, grid, faces, relax):
 
 
 def test_launch_counts():
-    a = _solver("D2Q5", 3, (40, 40), "pppppp", "magic")  # a small plane takes single steps
+    a = _solver("D2Q5", 3, (512, 512), "pppppp", "magic")  # a plane of middle size takes single steps
     assert [a.step_launches(n) for n in (0, 1, 2, 20, 71)] == [0, 1, 2, 20, 71]
-    b = _solver("D1Q3", 3, (500,), "pppppp", "magic")  # eight at a time, the last by itself
+    b = _solver("D1Q3", 3, (50000,), "pppppp", "magic")  # eight at a time, the last by itself
     assert [b.step_launches(n) for n in (1, 2, 9, 10, 20)] == [1, 2, 2, 3, 4]
     assert b.step_launches(71) == 1 + 2 * 4 + 1 + 1
