@@ -393,4 +393,92 @@ LBMS_HD bool collide_fixed(double (&f)[S][L::Q], const FixedTable& t)
     return true;
 }
 
+#ifdef __CUDACC__
+// collide_fixed of a ternary node by two lanes, one per species (own: this lane's, 0 or 1):
+// f holds that species' populations, and the lane 16 away holds the other's.  The same
+// integer operations per species, so the same results; the lanes exchange mole fractions
+// and departures by shuffles.  All lanes of the warp take part; false (in both lanes of
+// the node, f unchanged) where the node does not fit or is not active.
+template <typename L>
+__device__ __forceinline__ bool collide_fixed_lane(double (&f)[L::Q], const FixedTable& t, int own, bool active)
+{
+    using namespace fx;
+    constexpr int Q = L::Q;
+    constexpr unsigned all = 0xffffffffu;
+    uint32_t top = 0;
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+        const uint32_t h = (uint32_t)(bits_of(f[k]) >> 32) & 0x7fffffffu;
+        top = h > top ? h : top;
+    }
+    const Block e = block((int)(top >> 20), block_bits<L>());
+    bool fits = active && e.M <= 1022 && (e.M == 0 || e.M >= 120);
+    int64_t x[Q], sum = 0;
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+        x[k] = to_fixed(f[k], e, block_bits<L>(), (k & 1) != 0);
+        sum += x[k];
+    }
+    const int64_t half = sum >> 1, mine = to_abs(sum, e);
+    fits &= (uint64_t)(mine + kOne / 16) <= (uint64_t)(kOne + kOne / 8) && half < kLimit && half > -kLimit;
+    const int64_t other = __shfl_xor_sync(all, (long long)mine, 16);
+    const int64_t x3 = kOne - mine - other;
+    fits &= (uint64_t)(x3 + kOne / 16) <= (uint64_t)(kOne + kOne / 8);
+    const X a = split(x3), b = split(own ? other : mine), c = split(own ? mine : other);
+    const int64_t det = dot(a, t.det[0], b, t.det[1], c, t.det[2]);
+    const Cf n0 = own ? t.n22[0] : t.n11[0], n1 = own ? t.n22[1] : t.n11[1], n2 = own ? t.n22[2] : t.n11[2];
+    const int64_t n = dot(a, n0, b, n1, c, n2);
+    fits &= det > kOne / 32 && n > 0 && n < det;
+    const int up = fits ? clz64((uint64_t)det) - 2 : 0;
+    const int64_t y = reciprocal(fits ? det << up : int64_t(1) << 61);
+    const int64_t h = mul(split((n << up) >> 2), coef(y));
+    const Cf l1 = coef(h >> 2);
+    Cf l2 = l1;
+    if (!t.srt) {
+        const int64_t unit = int64_t(1) << 60;
+        l2 = coef(mul(split(unit - h), coef(reciprocal(4 * unit - h))) >> 2);
+    }
+    const int64_t p = mul(split(half), coef(mul(split(y << 1), own ? t.g2 : t.g1)));
+    const int more = up > 3 ? up - 3 : 0, less = up > 3 ? 0 : 3 - up;
+    const int64_t lim = kLimit >> more;
+    fits &= p < lim && p > -lim;
+    const X q = split((int64_t)((uint64_t)p << more) >> less);
+    const unsigned votes = __ballot_sync(all, fits);
+    const int lane = (int)(threadIdx.x & 31u);
+    fits = ((votes >> lane) & (votes >> (lane ^ 16)) & 1u) != 0;
+    if (votes == 0) return false;
+    int64_t rest = sum, even = 0;
+    int32_t off = 0;
+    double out[Q];
+#pragma unroll
+    for (int pr = 0; pr < L::NPAIR; ++pr) {
+        const int ka = L::K0 + 2 * pr, kb = ka + 1;
+        if (pr == 0 || L::w(ka) != L::w(ka - 1))
+            even = mul(split(half), coef((int64_t)(4.0 * L::w(ka) * 288230376151711744.0 + 0.5)));
+        const int64_t sym = x[ka] + x[kb] - even, asym = x[ka] - x[kb];
+        const Cf s1 = coef_of_abs(sym, e), a1 = coef_of_abs(asym, e);
+        const Cf s2 = {__shfl_xor_sync(all, s1.h, 16), __shfl_xor_sync(all, s1.l4, 16)};
+        const Cf a2 = {__shfl_xor_sync(all, a1.h, 16), __shfl_xor_sync(all, a1.l4, 16)};
+        const int64_t ds = dot(split(sym), l2, q, s2), da = dot(split(asym), l1, q, a2);
+        int32_t d;
+        if (ka != 0) {
+            const int64_t na = x[ka] - (ds + da);
+            out[ka] = to_double(na, e, d);
+            rest -= na;
+            off += d;
+        }
+        const int64_t nb = x[kb] - (ds - da);
+        out[kb] = to_double(nb, e, d);
+        rest -= nb;
+        off += d;
+    }
+    int32_t d;
+    out[0] = to_double(rest - off, e, d);
+    if (fits)
+#pragma unroll
+        for (int k = 0; k < Q; ++k) f[k] = out[k];
+    return fits;
+}
+#endif
+
 }  // namespace lbms

@@ -396,6 +396,50 @@ __global__ void __launch_bounds__(kBlock, StepOccupancy<LAT, S, T>::value) k_ste
     if (MASS) write_mass_partials<S>(xi, active, p.mass, lb);
 }
 
+// A plain step of a ternary FP64 grid with two lanes per node, one for each evolved
+// species: lanes 0 to 15 of a warp take the first species of 16 consecutive nodes, lanes
+// 16 to 31 the second.  On small grids a step waits for the dependent arithmetic of one
+// node; half of it per lane is half the wait.  The results are those of k_step.
+template <int LAT>
+__global__ void __launch_bounds__(kSmallBlock) k_step_species(StepParams<double> p)
+{
+    using L = Lattice<LAT>;
+    constexpr int Q = L::Q, S = 2;
+    const int own = (threadIdx.x >> 4) & 1;
+    const uint32_t slot = blockIdx.x * (kSmallBlock / 2) + (threadIdx.x >> 5) * 16 + (threadIdx.x & 15);
+    const bool active = slot < p.g.cells;
+    const uint32_t cell = active ? slot : p.g.cells - 1;
+    const Neighbourhood h = neighbourhood<L::DIM, false>(p.g, cell);
+    await_previous_grid();
+    const uint32_t step = *p.clock_in;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *p.clock_out = step + 1;
+    const size_t base = (size_t)own * Q * p.g.cells;
+    double f1[1][Q];
+    pull<LAT, 1, double, false, false, S>(p.fin + base, p.g, cell, h, f1, p.xb ? p.xb + own : nullptr);
+    double(&f)[Q] = f1[0];
+    const bool done = collide_fixed_lane<L>(f, p.fixed.table, own, active);
+    if (__any_sync(0xffffffffu, active && !done)) {
+        // a node of the warp takes the FP64 arithmetic, of both species in either lane
+        double both[S][Q], xi[S + 1], L1[S][S], L2[S][S];
+#pragma unroll
+        for (int k = 0; k < Q; ++k) {
+            const double o = __shfl_xor_sync(0xffffffffu, f[k], 16);
+            both[0][k] = own ? o : f[k];
+            both[1][k] = own ? f[k] : o;
+        }
+        if (active && !done) {
+            mole_fractions<LAT, S, double>(both, xi);
+            relaxation_matrices<S, double>(xi, p.co.invD, 1.0 / L::cs2(), p.relax, L1, L2);
+            collide<LAT, S, double>(both, xi, L1, L2, 0u);
+#pragma unroll
+            for (int k = 0; k < Q; ++k) f[k] = own ? both[1][k] : both[0][k];
+        }
+    }
+    if (active)
+#pragma unroll
+        for (int k = 0; k < Q; ++k) p.fout[base + (size_t)k * p.g.cells + cell] = f[k];
+}
+
 // Two nodes per thread (c, c + 1 with c even), for the lattices with Q <= 7 and
 // S <= 2 in FP32, whose per-node instruction count rather than HBM bandwidth
 // limits the one-node kernel: the pair's rest populations (if the lattice has a
@@ -554,6 +598,12 @@ __global__ void __launch_bounds__(kBlock / 2, MASS ? PairOccupancy<LAT, S, T>::m
 // Smallest grid stepped by the pair kernel: 2^21 nodes, whose populations
 // (at least 2 x 2 x 3 x 4 B per node) no longer fit the 129 MB L2.
 constexpr uint32_t kPairMinCells = 1u << 21;
+
+// Largest grid stepped with two lanes per node.  us per step, one lane -> two: D2Q5 100^2
+// 3.08 -> 2.73, 128^2 3.06 -> 2.88, 200^2 4.54 -> 4.38, D2Q9 300^2 11.7 -> 10.5, D3Q7
+// 24 x 16 x 12 3.79 -> 2.61; but D2Q5 400^2 11.4 -> 11.8, 1024^2 57 -> 69, D3Q7
+// 101 x 96 x 67 47 -> 53, where the duplicated matrix work counts.
+constexpr uint32_t kSpeciesMaxCells = 3u << 15;
 
 // Whether the pair kernel takes a step of this solver (see k_step_pair).
 template <int LAT, int S, typename T>
@@ -819,6 +869,11 @@ cudaError_t launch(Op op, const KArgs& a)
                     if (op == OP_STEP_MASS)
                         return launch_chained(k_step_pair<LAT, S, T, true>, blocks, kBlock / 2, a.stream, p);
                 }
+            }
+            if constexpr (S == 2 && sizeof(T) == 8) {
+                if (op == OP_STEP && a.fixed.on && a.cells <= kSpeciesMaxCells)
+                    return launch_chained(k_step_species<LAT>, (a.cells + kSmallBlock / 2 - 1) / (kSmallBlock / 2),
+                                          kSmallBlock, a.stream, p);
             }
             if (op == OP_STEP) return launch_chained(k_step<LAT, S, T, false, false>, blocks, tb, a.stream, p);
             if (op == OP_STEP_MASS) return launch_chained(k_step<LAT, S, T, true, false>, blocks, tb, a.stream, p);

@@ -439,7 +439,8 @@ __device__ __forceinline__ int link_wall(int k, const Neighbourhood& h)
 // a rest velocity, which never moves) itself.  SKIP_Y: the caller has loaded the
 // moving populations that do not move along x (the two-nodes-per-thread kernels
 // pair them); their Dirichlet correction below still applies.
-template <int LAT, int S, typename T, bool SKIP_REST = false, bool SKIP_Y = false>
+// XS: species in a row of xb (where f holds only some of them).
+template <int LAT, int S, typename T, bool SKIP_REST = false, bool SKIP_Y = false, int XS = S>
 __device__ __forceinline__ void pull(const T* __restrict__ fin, const Geom& g, uint32_t cell,
                                      const Neighbourhood& h, T (&f)[S][Lattice<LAT>::Q],
                                      const T* __restrict__ xb, const Halo<T>* halo = nullptr)
@@ -489,7 +490,7 @@ __device__ __forceinline__ void pull(const T* __restrict__ fin, const Geom& g, u
             const int wf = link_wall<LAT>(k, h);
             if (wf >= 0 && ((h.dir >> wf) & 1u)) {
 #pragma unroll
-                for (int s = 0; s < S; ++s) f[s][k] = T(2.0 * L::w(k)) * xb[wf * S + s] - f[s][k];
+                for (int s = 0; s < S; ++s) f[s][k] = T(2.0 * L::w(k)) * xb[wf * XS + s] - f[s][k];
             }
         }
     }
