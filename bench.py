@@ -661,7 +661,7 @@ def measure_batch(steps: int, warmup: int, local: int, count: int = BATCH_COUNT,
         else:
             b.set_schedule(schedule)
             chosen, tune_ms = schedule, []
-        launches_per_step = b.launches_per_step()
+        launches = b.step_launches(steps)
         x0_host = torch.empty(int(b.offsets[-1]), dtype=torch.float32).pin_memory()
         for i in range(count):
             x0_host[int(b.offsets[i]):int(b.offsets[i + 1])] = torch.from_numpy(
@@ -702,7 +702,7 @@ def measure_batch(steps: int, warmup: int, local: int, count: int = BATCH_COUNT,
             "l2": "state %.1f GB per step vs 129 MB L2" % (bytes_per_step / 1e9),
         },
         "roofline": roof,
-        "gpu_launches": steps * launches_per_step,
+        "gpu_launches": launches,
         "clocks": clocks,
         "status_flags": flags,
         "mass_drift_rel": float(np.max(np.abs(mass - mass0) / np.abs(mass0))),

@@ -508,9 +508,14 @@ int lbms_batch_get_schedule(const lbms_batch_t* b);
 
 /* Kernel launches one step takes under the current schedule (1 for the
  * streamed schedule, the number of instance groups otherwise); a call of
- * lbms_batch_step(n) launches n times this many step kernels and one mass
- * reduction.  -1 for a NULL handle. */
+ * lbms_batch_step(n) launches at most n times this many step kernels.  -1 for a
+ * NULL handle. */
 int lbms_batch_launches_per_step(const lbms_batch_t* b);
+
+/* Kernel launches that lbms_batch_step(b, n_steps) makes (or replays) under the
+ * current schedule: large planes take several steps per launch.  0 for
+ * n_steps < 1, -1 for a NULL handle. */
+long lbms_batch_step_launches(const lbms_batch_t* b, long n_steps);
 
 /*
  * Candidate tuner: times every candidate over trial_steps steps (after one

@@ -59,8 +59,29 @@ int lattice_dim(int lat)
     return lat == LBMS_D3Q7 || lat == LBMS_D3Q15 || lat == LBMS_D3Q6 ? 3 : (lat == LBMS_D1Q3 ? 1 : 2);
 }
 
+// Parts of a batch's passes of several steps (batch.cuh), or 0 where it takes single steps:
+// ternary and binary FP32 batches on D2Q4 and D2Q5 from 2^22 nodes.  A part has up to 96
+// rows, fewer (down to 16) in batches that would not give every SM enough warps.
+int part_rows(double nodes)
+{
+    const double r = nodes / (double)(1 << 18);
+    return r < 16.0 ? 16 : (r > 96.0 ? 96 : (int)r);
+}
+size_t count_parts(int lat, int n, int count, const int* grids, int dtype)
+{
+    if (dtype != LBMS_F32 || n > 3 || (lat != LBMS_D2Q5 && lat != LBMS_D2Q4)) return 0;
+    double nodes = 0.0, parts = 0.0;
+    for (int i = 0; i < count; ++i) nodes += (double)grids[3 * i] * grids[3 * i + 1];
+    if (nodes < (double)(1 << 22) || nodes > (double)(1 << 29)) return 0;
+    const int rows = part_rows(nodes);
+    for (int i = 0; i < count; ++i)
+        parts += ceil((double)grids[3 * i] / kBatchStrip) * ceil((double)grids[3 * i + 1] / rows);
+    return parts < 1e8 ? (size_t)parts : 0;
+}
+
 struct BLayout {
     uint32_t total_blocks = 0, total_nodes = 0;
+    size_t parts = 0, off_parts = 0;
     size_t f_bytes = 0, off_f1 = 0, off_partials = 0, off_mass = 0, off_inst = 0, off_blk = 0,
            off_invD = 0, off_clock = 0, off_foff = 0, off_xb = 0, off_fixed = 0, off_status = 0, off_staging = 0,
            staging_bytes = 0, total = 0;
@@ -99,7 +120,9 @@ bool batch_layout(int lat, int n, int count, const int* grids, int dtype, BLayou
     L->off_xb = L->off_foff + align_up((size_t)count * sizeof(long long));
     // Dirichlet compositions [count][6][S]
     L->off_fixed = L->off_xb + align_up((size_t)count * 6 * (n - 1) * es);
-    L->off_status = L->off_fixed + (dtype == LBMS_F64 ? align_up((size_t)count * sizeof(FixedTable)) : 0);
+    L->off_parts = L->off_fixed + (dtype == LBMS_F64 ? align_up((size_t)count * sizeof(FixedTable)) : 0);
+    L->parts = count_parts(lat, n, count, grids, dtype);
+    L->off_status = L->off_parts + align_up(L->parts * sizeof(BatchPart));
     L->off_staging = L->off_status + kAlign;
     // staging: large enough for the biggest instance's fields, at most 16 MiB beyond that
     const size_t biggest = (size_t)max_field * n * (1 + dim) * es;
@@ -161,6 +184,7 @@ struct lbms_batch_s {
     BatchInst* inst_dev = nullptr;
     uint32_t* blk_dev = nullptr;
     void* invD_dev = nullptr;
+    BatchPart* parts_dev = nullptr;       // parts of the passes of several steps
     FixedTable* fixed_dev = nullptr;      // [count] coefficients of the fixed-point collision (FP64)
     uint32_t* clock = nullptr;
     long long* foff_dev = nullptr;
@@ -247,6 +271,18 @@ cudaError_t bstep(const lbms_batch_t* b, int src, bool mass, uint32_t b0, uint32
     return bdispatch(b, mass ? BOP_STEP_MASS : BOP_STEP, a);
 }
 
+// Steps one pass of the streamed two-nodes-per-thread candidate takes: three where the batch
+// has parts and no Dirichlet faces, else one.  4096 D2Q5 ternary instances of 32^2 to 256^2,
+// 20 steps with their fields in and out: 27.35 -> 21.88 ms.
+int bdepth(const lbms_batch_t* b)
+{
+    return b->schedule == 0 && b->shape == 1 && b->lay.parts && !b->any_dirichlet ? kBatchDepth : 1;
+}
+
+// Launches a run of n plain steps of the streamed schedule takes (split evenly, as for
+// single solves).
+long bpasses(const lbms_batch_t* b, long n) { return (n + bdepth(b) - 1) / bdepth(b); }
+
 cudaError_t bfinalize(const lbms_batch_t* b, cudaStream_t st)
 {
     if (b->dtype == LBMS_F32)
@@ -300,13 +336,33 @@ int graph_steps(const lbms_batch_t* b)
     return b->schedule == 0 ? kStreamSteps : kCandidates[b->schedule].chunk;
 }
 
+// Whether launch_body(steps) leaves the state in the other buffer.
+bool run_parity(const lbms_batch_t* b, long steps)
+{
+    return ((b->schedule == 0 ? bpasses(b, steps) : steps) & 1) != 0;
+}
+
 cudaError_t launch_body(const lbms_batch_t* b, int parity, int steps, cudaStream_t st)
 {
     cudaError_t e = cudaSuccess;
     if (b->schedule == 0) {
-        int src = parity;
-        for (int i = 0; i < steps && e == cudaSuccess; ++i, src = 1 - src)
-            e = bstep(b, src, false, 0, b->lay.total_blocks, st);
+        int src = parity, left = steps;
+        for (long passes = bpasses(b, steps); passes > 0 && e == cudaSuccess; --passes, src = 1 - src) {
+            const int m = (int)((left + passes - 1) / passes);
+            if (m == 1) {
+                e = bstep(b, src, false, 0, b->lay.total_blocks, st);
+            } else {
+                BArgs a = bargs(b, st, 0, b->lay.total_blocks);
+                a.fin = b->f[src];
+                a.fout = b->f[1 - src];
+                a.parity = src;
+                a.parts = b->parts_dev;
+                a.nparts = (uint32_t)b->lay.parts;
+                a.steps = m;
+                e = bdispatch(b, BOP_ROWS, a);
+            }
+            left -= m;
+        }
         return e;
     }
     for (const auto& g : b->groups) {
@@ -422,6 +478,7 @@ int lbms_batch_create(lbms_batch_t** out, int lattice, int n_species, int count,
     b->foff_dev = reinterpret_cast<long long*>(b->ws + L.off_foff);
     b->xb_dev = b->ws + L.off_xb;
     b->fixed_dev = reinterpret_cast<FixedTable*>(b->ws + L.off_fixed);
+    b->parts_dev = reinterpret_cast<BatchPart*>(b->ws + L.off_parts);
     b->dirichlet.assign(count, 0u);
     b->xb_set.assign(count, 0u);
     b->status = reinterpret_cast<uint32_t*>(b->ws + L.off_status);
@@ -434,6 +491,11 @@ int lbms_batch_create(lbms_batch_t** out, int lattice, int n_species, int count,
     std::vector<uint32_t> blk(L.total_blocks);
     std::vector<char> invD((size_t)count * n * n * b->es);
     std::vector<FixedTable> fixed(dtype == LBMS_F64 ? count : 0);
+    std::vector<BatchPart> parts;
+    parts.reserve(L.parts);
+    double nodes = 0.0;
+    for (int c = 0; c < count; ++c) nodes += (double)grids[3 * c] * grids[3 * c + 1] * grids[3 * c + 2];
+    const int rows = part_rows(nodes);
     uint32_t block = 0;
     long long off = 0;
     for (int c = 0; c < count; ++c) {
@@ -460,6 +522,9 @@ int lbms_batch_create(lbms_batch_t** out, int lattice, int n_species, int count,
         d.pad = 0;
         for (uint32_t k = 0; k < d.nblocks; ++k) blk[block + k] = (uint32_t)c;
         block += d.nblocks;
+        for (int y = 0; L.parts && y < ka.ny; y += rows)
+            for (int strip = 0; strip * kBatchStrip < ka.nx; ++strip)
+                parts.push_back({(uint32_t)c, strip, y, y + rows < ka.ny ? y + rows : ka.ny});
         b->packed_off[c] = off;
         off += (long long)n * ka.cells;
         if (ka.cells > maxcells) maxcells = ka.cells;
@@ -495,6 +560,9 @@ int lbms_batch_create(lbms_batch_t** out, int lattice, int n_species, int count,
                             b->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b->invD_dev, invD.data(), invD.size(), cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess && L.parts)
+        e = cudaMemcpyAsync(b->parts_dev, parts.data(), parts.size() * sizeof(BatchPart), cudaMemcpyHostToDevice,
+                            b->stream);
     if (e == cudaSuccess && dtype == LBMS_F64)
         e = cudaMemcpyAsync(b->fixed_dev, fixed.data(), fixed.size() * sizeof(FixedTable), cudaMemcpyHostToDevice,
                             b->stream);
@@ -595,7 +663,7 @@ int lbms_batch_step(lbms_batch_t* b, long n_steps)
             }
             e = cudaGraphLaunch(b->graph[b->cur], b->stream);
             if (e != cudaSuccess) return bcuda(b, e, "cudaGraphLaunch");
-            if (gs & 1) b->cur = 1 - b->cur;
+            if (run_parity(b, gs)) b->cur = 1 - b->cur;
             body -= gs;
             b->steps += gs;
         }
@@ -604,7 +672,7 @@ int lbms_batch_step(lbms_batch_t* b, long n_steps)
         const int chunk = (int)(body < gs ? body : gs);
         e = launch_body(b, b->cur, chunk, b->stream);
         if (e != cudaSuccess) return bcuda(b, e, "batch step kernel");
-        if (chunk & 1) b->cur = 1 - b->cur;
+        if (run_parity(b, chunk)) b->cur = 1 - b->cur;
         body -= chunk;
         b->steps += chunk;
     }
@@ -772,6 +840,15 @@ int lbms_batch_launches_per_step(const lbms_batch_t* b)
 {
     if (!b) return -1;
     return b->schedule == 0 ? 1 : (int)b->groups.size();
+}
+
+long lbms_batch_step_launches(const lbms_batch_t* b, long n_steps)
+{
+    if (!b) return -1;
+    if (n_steps < 1) return 0;
+    if (b->schedule != 0) return (n_steps - 1) * (long)b->groups.size() + 1;
+    const long gs = graph_steps(b), body = n_steps - 1;
+    return body / gs * bpasses(b, gs) + bpasses(b, body % gs) + 1;
 }
 
 int lbms_batch_tune(lbms_batch_t* b, int trial_steps, double* ms_per_step, int* chosen)

@@ -9,6 +9,7 @@
 // for bit.
 #pragma once
 
+#include "fused.cuh"
 #include "kernels.cuh"
 
 namespace lbms {
@@ -22,7 +23,17 @@ struct BatchInst {
     uint32_t pad;
 };
 
-enum BatchOp : int { BOP_STEP = 0, BOP_STEP_MASS = 1, BOP_INIT = 2, BOP_MOMENTS = 3, BOP_MASS = 4 };
+enum BatchOp : int { BOP_STEP = 0, BOP_STEP_MASS = 1, BOP_INIT = 2, BOP_MOMENTS = 3, BOP_MASS = 4, BOP_ROWS = 5 };
+
+// The passes of several steps over a batch's planes (march_rows): a warp takes one part, rows
+// [y0, y1) of one strip of an instance.  One margin serves passes of two and three steps.
+constexpr int kBatchDepth = 3;
+constexpr int kBatchMargin = kBatchDepth - 1;
+constexpr int kBatchStrip = 32 - 2 * kBatchMargin;
+struct BatchPart {
+    uint32_t inst;
+    int strip, y0, y1;
+};
 
 // Everything a batched kernel may need, dtype-agnostic.
 struct BArgs {
@@ -49,6 +60,9 @@ struct BArgs {
     int nodes_per_thread = 1;                 // plain steps: 1 or 2 (k_batch_step_pair)
     const void* xb = nullptr;                 // [count][6][S] Dirichlet compositions
     bool dirichlet = false;                   // some instance has a Dirichlet face
+    const BatchPart* parts = nullptr;         // passes of several steps: the parts,
+    uint32_t nparts = 0;                      // how many,
+    int steps = 1;                            // and the steps taken
     cudaStream_t stream = nullptr;
 };
 
@@ -222,6 +236,28 @@ constexpr bool batch_pair_lattice()
     return Lattice<LAT>::Q <= 5 && S <= 2 && sizeof(T) == 4;
 }
 
+// Several steps of every instance in one pass (march_rows, see fused.cuh), with the
+// instance's own grid, diffusivities and step counter.
+template <int LAT, int S, int K>
+__global__ void __launch_bounds__(kFusedBlock, RowOccupancy<LAT, S>::value)
+    k_batch_rows(BatchParams<float> p, const BatchPart* __restrict__ parts, uint32_t nparts)
+{
+    const uint32_t at = blockIdx.x * (kFusedBlock / 32) + (threadIdx.x >> 5);
+    if (at >= nparts) return;
+    const BatchPart part = parts[at];
+    const Geom& geom = p.inst[part.inst].g;
+    const RowGrid grid = {geom.nx, geom.ny, geom.noflux, p.inst[part.inst].base, p.total_nodes};
+    uint32_t* clk = p.clock + 2 * part.inst;
+    const uint32_t step = clk[p.parity];
+    if (part.strip == 0 && part.y0 == 0 && (threadIdx.x & 31) == 0) clk[1 - p.parity] = step + K;
+    float invD[S + 1][S + 1];
+#pragma unroll
+    for (int i = 0; i <= S; ++i)
+#pragma unroll
+        for (int j = 0; j <= S; ++j) invD[i][j] = p.invD[((size_t)part.inst * (S + 1) + i) * (S + 1) + j];
+    march_rows<LAT, S, K, kBatchMargin>(p.fin, p.fout, grid, part.strip, part.y0, part.y1, step, p.relax, invD);
+}
+
 template <int LAT, int S, typename T>
 __global__ void __launch_bounds__(kBlock) k_batch_mass(BatchParams<T> p)
 {
@@ -352,6 +388,20 @@ cudaError_t batch_launch(BatchOp op, const BArgs& a)
     p.J_out = static_cast<T*>(a.field_J);
     p.field_off = a.field_off;
     const T* xb = static_cast<const T*>(a.xb);
+    if (op == BOP_ROWS) {
+        if constexpr (batch_pair_lattice<LAT, S, T>() && Lattice<LAT>::DIM == 2) {
+            const uint32_t n = (a.nparts + kFusedBlock / 32 - 1) / (kFusedBlock / 32);
+            if (a.steps == 3)
+                k_batch_rows<LAT, S, 3><<<n, kFusedBlock, 0, a.stream>>>(p, a.parts, a.nparts);
+            else if (a.steps == 2)
+                k_batch_rows<LAT, S, 2><<<n, kFusedBlock, 0, a.stream>>>(p, a.parts, a.nparts);
+            else
+                return cudaErrorInvalidValue;
+            return cudaGetLastError();
+        } else {
+            return cudaErrorInvalidValue;
+        }
+    }
     const uint32_t blocks = a.block_end - a.block_begin;
     if (blocks == 0) return cudaSuccess;
     switch (op) {

@@ -74,8 +74,10 @@ struct March {
     bool wlo, whi;  // walls at the ends
     __device__ __forceinline__ int place(int r) const  // layer in the grid's range
     {
-        if (wlo) return r < 0 ? 0 : (r >= n ? n - 1 : r);
-        return r < 0 ? r + n : (r >= n ? (r - n >= n ? (r - n) % n : r - n) : r);
+        if (r >= 0 && r < n) return r;
+        if (wlo) return r < 0 ? 0 : n - 1;
+        const int m = r % n;
+        return m < 0 ? m + n : m;
     }
     __device__ __forceinline__ int below(int y) const { return y == 0 ? (wlo ? 0 : n - 1) : y - 1; }
     __device__ __forceinline__ int above(int y) const { return y == n - 1 ? (whi ? y : 0) : y + 1; }
@@ -91,21 +93,30 @@ struct Strip {
     static constexpr int W = 32 - 2 * H;
 };
 
+// The grid a warp marches through: a plane of its own, or one of a batch's (whose nodes
+// begin at `base` of a common node space).
+struct RowGrid {
+    int nx, ny;
+    uint32_t noflux;
+    uint32_t base;
+    uint32_t stride;  // nodes of a population plane
+};
+
 struct RowLane {
-    uint32_t x0, xl, xr;  // the lane's column and its neighbours (wrapped, or clamped at walls)
+    uint32_t x0, xl, xr;  // base + the lane's column and its neighbours (wrapped, or clamped at walls)
     bool bl, br;          // the column lies at a wall on its left / right
     bool wall;            // some column of the warp does
 };
 
 // The gather of row y for the first step, from memory.  INNER: a row with both neighbours inside the grid.
 template <int LAT, int S, bool INNER>
-__device__ __forceinline__ void load_row(const FusedParams<S>& p, const RowLane& c, const March& m, int y,
-                                         float (&f)[S][Lattice<LAT>::Q])
+__device__ __forceinline__ void load_row(const float* __restrict__ fin, const RowGrid& g, const RowLane& c, const March& m,
+                                         int y, float (&f)[S][Lattice<LAT>::Q])
 {
     using L = Lattice<LAT>;
     constexpr int Q = L::Q;
     const bool blo = !INNER && m.wlo && y == 0, bhi = !INNER && m.whi && y == m.n - 1;
-    const uint32_t nx = (uint32_t)p.nx, row = (uint32_t)y * nx;
+    const uint32_t nx = (uint32_t)g.nx, row = (uint32_t)y * nx;
     const uint32_t rdn = INNER ? row - nx : (uint32_t)m.below(y) * nx, rup = INNER ? row + nx : (uint32_t)m.above(y) * nx;
 #pragma unroll
     for (int k = 0; k < Q; ++k) {
@@ -113,9 +124,9 @@ __device__ __forceinline__ void load_row(const FusedParams<S>& p, const RowLane&
         const bool by = (cy > 0 && blo) || (cy < 0 && bhi);  // the source lies across a y wall
         const uint32_t r = cy > 0 ? rdn : (cy < 0 ? rup : row);
         const uint32_t x = (cx == 0 || by) ? c.x0 : (cx > 0 ? c.xl : c.xr);
-        const float* base = p.fin + (size_t)(by ? opp<LAT>(k) : k) * p.cells;
+        const float* plane = fin + (size_t)(by ? opp<LAT>(k) : k) * g.stride;
 #pragma unroll
-        for (int s = 0; s < S; ++s) f[s][k] = at_bytes(base + (size_t)(s * Q) * p.cells, (r + x) * 4u);
+        for (int s = 0; s < S; ++s) f[s][k] = at_bytes(plane + (size_t)(s * Q) * g.stride, (r + x) * 4u);
     }
     if (c.wall) {  // bounce-back at the walls along x: the node's own opposite population
 #pragma unroll
@@ -124,7 +135,7 @@ __device__ __forceinline__ void load_row(const FusedParams<S>& p, const RowLane&
             if (L::cx(k) > 0 ? c.bl : c.br)
 #pragma unroll
                 for (int s = 0; s < S; ++s)
-                    f[s][k] = at_bytes(p.fin + (size_t)(s * Q + opp<LAT>(k)) * p.cells, (row + c.x0) * 4u);
+                    f[s][k] = at_bytes(fin + (size_t)(s * Q + opp<LAT>(k)) * g.stride, (row + c.x0) * 4u);
         }
     }
 }
@@ -211,44 +222,40 @@ struct RowOccupancy {
     static constexpr int value = S >= 4 ? 2 : Lattice<LAT>::Q <= 5 ? (S == 3 ? 4 : 3) : (S == 1 ? 5 : (S == 2 ? 4 : 3));
 };
 
-template <int LAT, int S, int K>
-__global__ void __launch_bounds__(kFusedBlock, RowOccupancy<LAT, S>::value) k_fused_rows(FusedParams<S> p)
+// K steps of the rows [y0, y1) of one strip of W columns, with margins of H (at least K - 1).
+template <int LAT, int S, int K, int H, typename InvD>
+__device__ __forceinline__ void march_rows(const float* __restrict__ fin, float* __restrict__ fout, const RowGrid& grid,
+                                           int strip, int y0, int y1, uint32_t step, int relax, const InvD& invD)
 {
     using L = Lattice<LAT>;
-    constexpr int Q = L::Q;
-    constexpr int H = Strip<K>::H, W = Strip<K>::W;
-    static_assert(L::DIM == 2, "rows march along y");
-    await_previous_grid();
-    const uint32_t step = *p.clock_in;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *p.clock_out = step + K;
-    const uint32_t part = blockIdx.x * (kFusedBlock / 32) + (threadIdx.x >> 5);
+    constexpr int Q = L::Q, W = 32 - 2 * H;
+    static_assert(L::DIM == 2 && H >= K - 1, "rows march along y");
     const int lane = threadIdx.x & 31;
-    const int strip = (int)(part % (uint32_t)p.strips), seg = (int)(part / (uint32_t)p.strips);
-    if (seg >= p.segments) return;
-    const int nx = p.nx, ny = p.ny;
+    const int nx = grid.nx, ny = grid.ny;
     const int X = strip * W - H + lane;  // the lane's column; beyond the grid's edges wrapped or clamped
     RowLane c;
+    uint32_t x;
     {
-        const bool wl = p.noflux & 1u, wr = p.noflux & 2u;
-        auto place = [&](int x) -> uint32_t {
-            if (wl) return (uint32_t)(x < 0 ? 0 : (x >= nx ? nx - 1 : x));
-            const int m = x % nx;
-            return (uint32_t)(m < 0 ? m + nx : m);
+        const bool wl = grid.noflux & 1u, wr = grid.noflux & 2u;
+        auto place = [&](int v) -> uint32_t {
+            if (wl) return (uint32_t)(v < 0 ? 0 : (v >= nx ? nx - 1 : v));
+            const int r = v % nx;
+            return (uint32_t)(r < 0 ? r + nx : r);
         };
-        c.x0 = place(X);
-        c.xl = place(X - 1);
-        c.xr = place(X + 1);
+        x = place(X);
+        c.x0 = grid.base + x;
+        c.xl = grid.base + place(X - 1);
+        c.xr = grid.base + place(X + 1);
         c.bl = wl && X == 0;
         c.br = wr && X == nx - 1;
         c.wall = __any_sync(0xffffffffu, c.bl || c.br);
     }
     const bool mine = lane >= H && lane < 32 - H && X < nx;
-    const March m = {ny, (p.noflux & 4u) != 0, (p.noflux & 8u) != 0};
-    const uint32_t C = 0x27d4eb2du, rowC = (uint32_t)nx * C, key0 = c.x0 * C;
+    const March m = {ny, (grid.noflux & 4u) != 0, (grid.noflux & 8u) != 0};
+    const uint32_t C = 0x27d4eb2du, rowC = (uint32_t)nx * C, key0 = x * C;
     uint32_t hk[K];
 #pragma unroll
     for (int l = 0; l < K; ++l) hk[l] = mix32((step + l) * 0x9e3779b9u);
-    const int y0 = seg * p.rows, y1 = y0 + p.rows < ny ? y0 + p.rows : ny;  // the part's rows
     RowQueue<LAT, S> queue[K - 1];
     float nxt[S][Q];
     // Iteration j: the first step forms row y0 - (K - 1) + j, step l the row l below it.
@@ -261,7 +268,7 @@ __global__ void __launch_bounds__(kFusedBlock, RowOccupancy<LAT, S>::value) k_fu
         for (int s = 0; s < S; ++s)
 #pragma unroll
             for (int k = 0; k < Q; ++k) f[s][k] = nxt[s][k];
-        load_row<LAT, S, STEADY>(p, c, m, STEADY ? r0 + 1 : m.place(r0 + 1), nxt);
+        load_row<LAT, S, STEADY>(fin, grid, c, m, STEADY ? r0 + 1 : m.place(r0 + 1), nxt);
 #pragma unroll
         for (int l = 0; l < K; ++l) {
             const int r = r0 - l, y = STEADY ? r : m.place(r);
@@ -275,7 +282,7 @@ __global__ void __launch_bounds__(kFusedBlock, RowOccupancy<LAT, S>::value) k_fu
                 queue[l - 1].template complete<!STEADY>(f, c, m.whi && r == ny - 1, g);
                 queue[l - 1].template push<!STEADY>(f, c, m.wlo && r + 1 == 0);
             }
-            fused_node<LAT, S, float>(g, p.co.invD, p.relax, hk[l] ^ ((uint32_t)y * rowC + key0));
+            fused_node<LAT, S, float>(g, invD, relax, hk[l] ^ ((uint32_t)y * rowC + key0));
 #pragma unroll
             for (int s = 0; s < S; ++s)
 #pragma unroll
@@ -285,7 +292,7 @@ __global__ void __launch_bounds__(kFusedBlock, RowOccupancy<LAT, S>::value) k_fu
 #pragma unroll
                 for (int s = 0; s < S; ++s)
 #pragma unroll
-                    for (int k = 0; k < Q; ++k) at_bytes(p.fout + (size_t)(s * Q + k) * p.cells, at) = f[s][k];
+                    for (int k = 0; k < Q; ++k) at_bytes(fout + (size_t)(s * Q + k) * grid.stride, at) = f[s][k];
             }
         }
     };
@@ -294,7 +301,7 @@ __global__ void __launch_bounds__(kFusedBlock, RowOccupancy<LAT, S>::value) k_fu
     // loaded ahead is at most ny - 2
     const int s0 = y0 > 1 ? 2 * (K - 1) : 2 * K - 1 - y0;
     const int s1 = count - 1 < ny - 4 + K - y0 ? count - 1 : ny - 4 + K - y0;
-    load_row<LAT, S, false>(p, c, m, m.place(y0 - (K - 1)), nxt);
+    load_row<LAT, S, false>(fin, grid, c, m, m.place(y0 - (K - 1)), nxt);
     int j = 0;
     while (j < count) {
         if (j >= s0 && j <= s1) {
@@ -305,6 +312,20 @@ __global__ void __launch_bounds__(kFusedBlock, RowOccupancy<LAT, S>::value) k_fu
             ++j;
         }
     }
+}
+
+template <int LAT, int S, int K>
+__global__ void __launch_bounds__(kFusedBlock, RowOccupancy<LAT, S>::value) k_fused_rows(FusedParams<S> p)
+{
+    await_previous_grid();
+    const uint32_t step = *p.clock_in;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *p.clock_out = step + K;
+    const uint32_t part = blockIdx.x * (kFusedBlock / 32) + (threadIdx.x >> 5);
+    const int strip = (int)(part % (uint32_t)p.strips), seg = (int)(part / (uint32_t)p.strips);
+    if (seg >= p.segments) return;
+    const int y0 = seg * p.rows, y1 = y0 + p.rows < p.ny ? y0 + p.rows : p.ny;  // the part's rows
+    const RowGrid grid = {p.nx, p.ny, p.noflux, 0u, p.cells};
+    march_rows<LAT, S, K, K - 1>(p.fin, p.fout, grid, strip, y0, y1, step, p.relax, p.co.invD);
 }
 
 // Lines (1D): a warp takes kLineBlocks runs of 32 consecutive nodes, a lane one node of

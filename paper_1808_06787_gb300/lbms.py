@@ -45,7 +45,7 @@ EXPORTED = (
     "lbms_batch_workspace_size", "lbms_batch_create", "lbms_batch_set_state", "lbms_batch_step",
     "lbms_batch_moments", "lbms_batch_mass", "lbms_batch_status", "lbms_batch_set_boundary",
     "lbms_batch_set_schedule",
-    "lbms_batch_get_schedule", "lbms_batch_launches_per_step", "lbms_batch_tune",
+    "lbms_batch_get_schedule", "lbms_batch_launches_per_step", "lbms_batch_step_launches", "lbms_batch_tune",
     "lbms_batch_steps_done",
     "lbms_batch_last_error", "lbms_batch_destroy",
     "lbms_get_state", "lbms_set_state_raw", "lbms_recompute", "lbms_adjoint_scratch_size",
@@ -161,6 +161,8 @@ def load(build_if_missing: bool = True) -> ctypes.CDLL:
         L.lbms_batch_get_schedule.restype = I
         L.lbms_batch_launches_per_step.argtypes = [P]
         L.lbms_batch_launches_per_step.restype = I
+        L.lbms_batch_step_launches.argtypes = [P, ctypes.c_long]
+        L.lbms_batch_step_launches.restype = ctypes.c_long
         L.lbms_batch_tune.argtypes = [P, I, P, P]
         L.lbms_batch_tune.restype = I
         L.lbms_batch_steps_done.argtypes = [P]
@@ -670,6 +672,10 @@ class BatchSolver:
     def launches_per_step(self) -> int:
         """Step-kernel launches per step under the current schedule."""
         return int(load().lbms_batch_launches_per_step(self._h))
+
+    def step_launches(self, n: int) -> int:
+        """Kernel launches that ``step(n)`` makes under the current schedule."""
+        return int(load().lbms_batch_step_launches(self._h, int(n)))
 
     def tune(self, trial_steps: int = 32):
         """Time every step candidate (schedule x kernel shape) and keep the fastest

@@ -104,3 +104,38 @@ def test_launch_counts():
     b = _solver("D1Q3", 3, (50000,), "pppppp", "magic")  # eight at a time, the last by itself
     assert [b.step_launches(n) for n in (1, 2, 9, 10, 20)] == [1, 2, 2, 3, 4]
     assert b.step_launches(71) == 1 + 2 * 4 + 1 + 1
+
+
+@pytest.mark.parametrize("lattice,n", [("D2Q5", 3), ("D2Q5", 2), ("D2Q4", 3)])
+@pytest.mark.parametrize("relax", ["magic", "srt"])
+def test_fused_batches_equal_single_steps(lattice, n, relax):
+    """A batch large enough for passes of several steps, with instances of every awkward
+    shape in it, under the streamed candidate (passes) and the one-node candidate (single
+    steps), over runs that leave remainders: fields, fluxes and masses are equal bit for bit."""
+    from paper_1808_06787_gb300 import BatchSolver
+
+    grids = [(1, 1), (2, 1), (1, 2), (33, 17), (50, 3), (5, 91), (28, 96), (29, 97), (56, 193), (257, 3)]
+    grids += [(251 - i, 240 + i) for i in range(72)]
+    assert sum(a * b for a, b in grids) >= 1 << 22
+    kinds = [("periodic",) * 6, ("noflux", "noflux") + ("periodic",) * 4, ("periodic",) * 2 + ("noflux",) * 2 + ("periodic",) * 2,
+             ("noflux",) * 4 + ("periodic",) * 2]
+    bcs = [kinds[i % 4] for i in range(len(grids))]
+    Ds = [sy.random_D(n, seed=100 + i) for i in range(len(grids))]
+    b = BatchSolver(lattice, Ds, grids, bcs=bcs, relax=relax)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    fields = []
+    for nx, ny in grids:
+        x = torch.rand((n, 1, ny, nx), device="cuda", dtype=torch.float64, generator=g) + 0.05
+        fields.append((x / x.sum(0, keepdim=True)).float())
+    got = {}
+    for candidate in (7, 0):
+        b.set_schedule(candidate)
+        b.set_state(b.pack(fields))
+        for steps in (1, 2, 3, 20, 40):
+            launches = b.step_launches(steps)
+            assert launches == steps if candidate == 0 or steps < 3 else launches < steps
+            b.step(steps)
+        x, J = b.moments(flux=True)
+        got[candidate] = (x, J, b.mass(), b.steps_done)
+    assert torch.equal(got[7][0], got[0][0]) and torch.equal(got[7][1], got[0][1])
+    assert np.array_equal(got[7][2], got[0][2]) and got[7][3] == got[0][3] == 66
