@@ -457,11 +457,17 @@ constexpr int fused_limit()
 }
 
 // Cuts n rows into parts of at least `least` rows: `wave` parts (per strip) fill the chip
-// once, and up to four waves are taken while a part keeps `good` rows.
-inline void cut(int n, double wave, int good, int least, int& segments, int& rows)
+// once.  Warps take different times, so two waves are taken while a part keeps `pair` rows
+// and up to four while it keeps `good`; but a part also forms 2 (K - 1) rows for its
+// neighbours.  D2Q5 ternary, us per step with one wave -> two: 1448^2 24.4 -> 20.4,
+// 2048 x 1100 28.5 -> 22.6, 3474 x 1576 69.5 -> 53.5 (single steps 27.7, 27.6, 65.2);
+// D2Q9 ternary 3402 x 1784 93.6 -> 86.4, but 2048^2 (31 rows) 56.5 -> 59.0, and with five
+// species, whose parts hold more, 129.9 -> 132.6.
+inline void cut(int n, double wave, int pair, int good, int least, int& segments, int& rows)
 {
     int waves = (int)((n / good) / wave);
-    waves = waves < 1 ? 1 : (waves > 4 ? 4 : waves);
+    waves = waves > 4 ? 4 : waves;
+    if (waves < 2) waves = n / pair >= 2.0 * wave ? 2 : 1;
     int s = (int)(waves * wave);
     if (s > n / least) s = n / least;
     if (s < 1) s = 1;
@@ -474,9 +480,8 @@ cudaError_t launch_rows(FusedParams<S>& p, const KArgs& a)
 {
     p.strips = (a.nx + Strip<K>::W - 1) / Strip<K>::W;
     const double resident = (double)a.sms * RowOccupancy<LAT, S>::value * (kFusedBlock / 32);
-    // several waves of warps even out their different speeds, but short parts pay for the
-    // 2 (K - 1) rows each forms for its neighbours
-    cut(a.ny, resident / p.strips, 80, 4 * K, p.segments, p.rows);
+    constexpr int pair = Lattice<LAT>::Q <= 5 ? 16 : (S <= 2 ? 32 : 80), good = Lattice<LAT>::Q <= 5 || S <= 2 ? 48 : 80;
+    cut(a.ny, resident / p.strips, pair, good, 4 * K, p.segments, p.rows);
     const uint32_t parts = (uint32_t)p.strips * (uint32_t)p.segments;
     return launch_chained(k_fused_rows<LAT, S, K>, (parts + 3) / 4, kFusedBlock, a.stream, p);
 }

@@ -9,8 +9,10 @@ import numpy as np
 import pytest
 
 
-def cut(n, wave, good, least):
-    waves = min(max(int((n // good) / wave), 1), 4)
+def cut(n, wave, pair, good, least):
+    waves = min(int((n // good) / wave), 4)
+    if waves < 2:
+        waves = 2 if n // pair >= 2.0 * wave else 1
     s = max(min(int(waves * wave), n // least), 1)
     rows = -(-n // s)
     return -(-n // rows), rows
@@ -18,14 +20,15 @@ def cut(n, wave, good, least):
 
 @pytest.mark.parametrize("steps", [2, 3])
 @pytest.mark.parametrize("blocks", [2, 3, 4, 5])
-def test_planes_are_covered_once(steps, blocks):
+@pytest.mark.parametrize("pair,good", [(16, 48), (32, 48), (80, 80)])
+def test_planes_are_covered_once(steps, blocks, pair, good):
     W, H = 32 - 2 * (steps - 1), steps - 1
     g = np.random.default_rng(steps * 10 + blocks)
     shapes = [(56, 24), (56, 1 << 20), (1 << 20, 24), (4095, 4097), (8192, 8192), (28, 2000)]
     shapes += [tuple(int(v) for v in np.exp(g.uniform(np.log(24), np.log(40000), 2))) for _ in range(200)]
     for nx, ny in shapes:
         strips = -(-nx // W)
-        segments, rows = cut(ny, 152 * blocks * 4 / strips, 80, 4 * steps)
+        segments, rows = cut(ny, 152 * blocks * 4 / strips, pair, good, 4 * steps)
         cols = np.zeros(nx, dtype=int)
         for t in {0, 1, strips // 2, strips - 2, strips - 1} if strips > 6 else range(strips):
             X = t * W - H + np.arange(32)
