@@ -60,8 +60,11 @@ int lattice_dim(int lat)
 }
 
 // Parts of a batch's passes of several steps (batch.cuh), or 0 where it takes single steps:
-// ternary and binary FP32 batches on D2Q4 and D2Q5 from 2^22 nodes.  A part has up to 96
-// rows, fewer (down to 16) in batches that would not give every SM enough warps.
+// ternary and binary FP32 batches on D2Q4 and D2Q5 from 2^22 nodes whose parts form at most
+// 1.6 times the batch's nodes, margins and idle lanes included.  A part has up to 96 rows,
+// fewer (down to 16) in batches that would not give every SM enough warps.  us per step,
+// single -> passes: 150 instances of 60^2 to 200^2 (1.5 times) 38.0 -> 36.3, but 1000 of 40^2
+// to 70^2 (1.8) 42.7 -> 47.4 and 2000 of 16^2 to 64^2 (2.2) 49.4 -> 58.8.
 int part_rows(double nodes)
 {
     const double r = nodes / (double)(1 << 18);
@@ -74,9 +77,13 @@ size_t count_parts(int lat, int n, int count, const int* grids, int dtype)
     for (int i = 0; i < count; ++i) nodes += (double)grids[3 * i] * grids[3 * i + 1];
     if (nodes < (double)(1 << 22) || nodes > (double)(1 << 29)) return 0;
     const int rows = part_rows(nodes);
-    for (int i = 0; i < count; ++i)
-        parts += ceil((double)grids[3 * i] / kBatchStrip) * ceil((double)grids[3 * i + 1] / rows);
-    return parts < 1e8 ? (size_t)parts : 0;
+    double formed = 0.0;
+    for (int i = 0; i < count; ++i) {
+        const double strips = ceil((double)grids[3 * i] / kBatchStrip), cuts = ceil((double)grids[3 * i + 1] / rows);
+        parts += strips * cuts;
+        formed += 32.0 * strips * (grids[3 * i + 1] + 2 * kBatchMargin * cuts);
+    }
+    return parts < 1e8 && formed <= 1.6 * nodes ? (size_t)parts : 0;
 }
 
 struct BLayout {
