@@ -259,9 +259,10 @@ def fp64_peak_tflops(sms: int, sm_mhz: float) -> float:
 
 
 def fp64_roofline(wl: "Workload", step_ms: float, sms: int, sm_mhz: float) -> dict:
-    """ALU roofline of the L2-resident FP64 workload: its step kernel is bound by the
-    FP64 pipes (57 % of their issue slots busy under ncu), not by HBM.  The peak
-    uses the device's SM count and the SM clock sampled while it ran."""
+    """ALU roofline of the L2-resident FP64 workload: the FP64 operations of the model's
+    collision against the FP64 pipes' peak (the device's SM count and the SM clock
+    sampled while it ran).  The step kernel does most of them in 64-bit fixed point on
+    the integer pipes and is bound by the latency of a step, not by HBM."""
     flops = D2Q5_TERNARY_FP64_FLOPS_PER_NODE * wl.cells
     achieved = flops / (step_ms * 1e-3) / 1e12
     peak = fp64_peak_tflops(sms, sm_mhz)
@@ -275,7 +276,8 @@ def fp64_roofline(wl: "Workload", step_ms: float, sms: int, sm_mhz: float) -> di
         "peak_source": "derived: %d SMs x %d DFMA/clk x 2 flops x %.0f MHz (sampled SM clock; FP64 pipe)"
                        % (sms, DFMA_PER_SM_CLK, sm_mhz),
         "algorithmic_flops_per_launch": flops,
-        "note": "FP64 flops per node counted by ncu on this kernel; state L2-resident",
+        "note": "FP64 flops per node of the collision in FP64 arithmetic (counted by ncu); done "
+                "in fixed point on the integer pipes; state L2-resident",
     }
 
 
@@ -416,8 +418,12 @@ def single_line(wl: Workload, m: dict, steps: int, world: int, t_ms: float, sms:
     glups = job_rate(float(wl.S) * wl.cells * steps, world, t_ms) / 1e9
     bytes_per_launch = 2.0 * wl.S * wl.Q * wl.es * wl.cells
     state_gb = bytes_per_launch / 1e9
+    launches = m.get("launches", steps)  # large planes and lines take several steps per launch
     roof = (fp64_roofline(wl, t_ms / steps, sms, sm_mhz) if wl.key == "sine"
-            else hbm_roofline(bytes_per_launch, t_ms / steps, measured_traffic(wl)))
+            else hbm_roofline(bytes_per_launch, t_ms / launches, measured_traffic(wl)))
+    if launches < steps and wl.key != "sine":
+        roof["note"] = ("%d steps in %d launches: each reads and writes the state once; bound by the "
+                        "issue rate rather than by HBM" % (steps, launches))
     return {
         "value": round(glups, 4),
         "unit": "GLUPS",
@@ -441,7 +447,7 @@ def single_line(wl: Workload, m: dict, steps: int, world: int, t_ms: float, sms:
                   % (state_gb * 1e3)),
         },
         "roofline": roof,
-        "gpu_launches": m.get("launches", steps),
+        "gpu_launches": launches,
         "status_flags": m["status_flags"],
         "mass_drift_rel": m["mass_drift_rel"],
     }
@@ -678,10 +684,12 @@ def measure_batch(steps: int, warmup: int, local: int, count: int = BATCH_COUNT,
         mass = b.mass()
     nodes = float(sum(int(g[0]) * int(g[1]) for g in grids))
     bytes_per_step = 2.0 * 2 * 5 * 4 * nodes
-    roof = hbm_roofline(bytes_per_step, ms / steps,
+    passes = launches if chosen % 7 == 0 else steps
+    roof = hbm_roofline(bytes_per_step, ms / passes,
                         recorded_traffic("traffic_batch_d2q5_4096_f32.json", [count, int(chosen)])
                         if chosen % 7 == 0 else None)
-    roof["note"] = "algorithmic bytes of a streamed step; L2-blocked schedules move less"
+    roof["note"] = ("algorithmic bytes of a streamed launch (%d steps in %d launches); L2-blocked "
+                    "schedules move less" % (steps, passes))
     out = {
         "value": round(count * steps / BATCH_SOLVE_STEPS / (ms * 1e-3), 3),
         "unit": "solves/s",

@@ -430,7 +430,7 @@ cudaError_t launch_finalize(const lbms_t* h, cudaStream_t st)
 }
 
 // Most steps one launch takes (fused.cuh): the lattice's limit on grids where a pass over
-// several steps beats as many single steps.  Same-box times of 60-step calls, single ->
+// several steps beats as many single steps.  Times of 60-step calls, single ->
 // fused: D2Q5 ternary 1448^2 27.6 -> 24.9 us per step, 1024^2 14.0 -> 13.7 and 4096 x 300
 // 16.1 -> 16.2 (hence the higher line for it), 4096^2 194 -> 138; binary 1024^2 8.4 -> 6.0;
 // D2Q9 ternary 1024^2 23.1 -> 18.8, 724^2 11.1 -> 14.5; five species 724^2 24.3 -> 21.2;
@@ -451,7 +451,7 @@ int fused_depth(const lbms_t* h)
 
 // Most steps a tiled pass takes (tile.cuh), and its tile; 1 where single steps are faster:
 // above these sizes the margins, formed by several blocks, cost more than the waits they
-// save.  Same-box times, us per step, single -> tiled: FP32 D2Q5 ternary 48 x 40 1.73 ->
+// save.  Times, us per step, single -> tiled: FP32 D2Q5 ternary 48 x 40 1.73 ->
 // 0.77, 128^2 1.77 -> 0.91, 200^2 2.03 -> 1.61, 256^2 2.09 -> 1.88, D2Q9 128^2 2.01 -> 1.16,
 // four species 128^2 1.95 -> 1.15 and 200^2 2.23 -> 2.16, binary 256^2 2.13 -> 1.24; D3Q7
 // 24 x 16 x 12 1.79 -> 1.33, 28 x 24 x 16 1.95 -> 1.63, 40 x 24 x 24 2.08 -> 2.10 (single);
