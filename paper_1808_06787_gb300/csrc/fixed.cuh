@@ -29,9 +29,9 @@
 // sums of positive terms without cancellation.  For binary mixtures both matrices are
 // constants.
 //
-// A node whose numbers do not fit (a population of one or more, a mole fraction outside
-// [-1/16, 17/16], a magnitude below 2^-900, infinities, NaN) takes the FP64 arithmetic of
-// node.cuh; so does a solver whose diffusivities spread too far for the bits above
+// A node whose numbers do not fit (a population of one or more, in ternary mixtures a
+// moving one of a half or more, a mole fraction outside [-1/16, 17/16], a magnitude below
+// 2^-900, infinities, NaN) takes the FP64 arithmetic of node.cuh; so does a solver whose diffusivities spread too far for the bits above
 // (fixed_table).  The functions are plain integer C++, the same on the host.
 #pragma once
 
@@ -158,6 +158,23 @@ constexpr int block_bits()
     return L::Q == 9 ? 59 : 58;
 }
 
+// Bounds of a ternary node's numbers.  The departures of one species enter the other's
+// results as coefficients, below two in magnitude in units of 2^-58 of one, and every result
+// has to stay below 2^63.  With moving populations below a half (exponent field 1021) the even
+// and odd departures are below 1 + 2 w (17/16) <= 1.54 and 1, and with the sum below 2^62 and
+// Lambda_12/2 below 2^61 in the species' units, for the weights of each lattice
+//   |f_k| + |even| lambda_2/2 + |odd| Lambda_1/2 + |Lambda_12/2| (1.54 + 1)  < 7.5 2^60,
+//   |f_0| + 2 |w_0 sum - f_0| lambda_2/2 + 2 |Lambda_12/2| |w_0 xi - f_0|    < 7.5 2^60
+// (f_0: the rest population).  On D2Q9, whose numbers have one bit more, the rest
+// population takes part in the limit and the sum is below 2^61 (at equilibrium it is 2.25 of
+// the largest population, 2^60.2).
+template <typename L>
+LBMS_HD bool fits_pair(uint32_t rest, uint32_t moving, int64_t half)
+{
+    if (block_bits<L>() == 58) return (int)(moving >> 20) <= 1021;
+    return (int)((rest > moving ? rest : moving) >> 20) <= 1021 && half < kLimit / 2 && half > -kLimit / 2;
+}
+
 LBMS_HD Block block(int M, int bits)
 {
     const int r = 965 + bits - M;
@@ -279,12 +296,14 @@ LBMS_HD bool collide_fixed(double (&f)[S][L::Q], const FixedTable& t)
     bool fits = true;
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-        uint32_t top = 0;
+        uint32_t rest = 0, moving = 0;
 #pragma unroll
         for (int k = 0; k < Q; ++k) {
             const uint32_t h = (uint32_t)(bits_of(f[s][k]) >> 32) & 0x7fffffffu;
-            top = h > top ? h : top;
+            uint32_t& most = k < L::K0 ? rest : moving;
+            most = h > most ? h : most;
         }
+        const uint32_t top = rest > moving ? rest : moving;
         e[s] = block((int)(top >> 20), block_bits<L>());
         fits &= e[s].M <= 1022 && (e[s].M == 0 || e[s].M >= 120);
         int64_t a = 0;
@@ -297,6 +316,7 @@ LBMS_HD bool collide_fixed(double (&f)[S][L::Q], const FixedTable& t)
         sum[s] = a;
         xi[s] = to_abs(a, e[s]);
         fits &= half[s] < kLimit && half[s] > -kLimit;
+        if (S == 2) fits &= fits_pair<L>(rest, moving, half[s]);
         fits &= (uint64_t)(xi[s] + kOne / 16) <= (uint64_t)(kOne + kOne / 8);
     }
     Cf l1[S], l2[S];
@@ -339,12 +359,12 @@ LBMS_HD bool collide_fixed(double (&f)[S][L::Q], const FixedTable& t)
         q2 = split(r2);
     }
     if (!fits) return false;
-    int64_t rest[S];  // what the moving populations leave of the sums
+    uint64_t rest[S];  // what the moving populations leave of the sums (modulo 2^64 on the way)
     int32_t off[S];
     int64_t even[S];  // 2 w xi of the current weight
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-        rest[s] = sum[s];
+        rest[s] = (uint64_t)sum[s];
         off[s] = 0;
     }
 #pragma unroll
@@ -376,19 +396,19 @@ LBMS_HD bool collide_fixed(double (&f)[S][L::Q], const FixedTable& t)
             if (ka != 0) {
                 const int64_t na = x[s][ka] - (ds[s] + da[s]);
                 f[s][ka] = to_double(na, e[s], d);
-                rest[s] -= na;
+                rest[s] -= (uint64_t)na;
                 off[s] += d;
             }
             const int64_t nb = x[s][kb] - (ds[s] - da[s]);
             f[s][kb] = to_double(nb, e[s], d);
-            rest[s] -= nb;
+            rest[s] -= (uint64_t)nb;
             off[s] += d;
         }
     }
 #pragma unroll
     for (int s = 0; s < S; ++s) {
         int32_t d;
-        f[s][0] = to_double(rest[s] - off[s], e[s], d);
+        f[s][0] = to_double((int64_t)rest[s] - off[s], e[s], d);
     }
     return true;
 }
@@ -405,12 +425,14 @@ __device__ __forceinline__ bool collide_fixed_lane(double (&f)[L::Q], const Fixe
     using namespace fx;
     constexpr int Q = L::Q;
     constexpr unsigned all = 0xffffffffu;
-    uint32_t top = 0;
+    uint32_t still = 0, moving = 0;
 #pragma unroll
     for (int k = 0; k < Q; ++k) {
         const uint32_t h = (uint32_t)(bits_of(f[k]) >> 32) & 0x7fffffffu;
-        top = h > top ? h : top;
+        uint32_t& most = k < L::K0 ? still : moving;
+        most = h > most ? h : most;
     }
+    const uint32_t top = still > moving ? still : moving;
     const Block e = block((int)(top >> 20), block_bits<L>());
     bool fits = active && e.M <= 1022 && (e.M == 0 || e.M >= 120);
     int64_t x[Q], sum = 0;
@@ -421,6 +443,7 @@ __device__ __forceinline__ bool collide_fixed_lane(double (&f)[L::Q], const Fixe
     }
     const int64_t half = sum >> 1, mine = to_abs(sum, e);
     fits &= (uint64_t)(mine + kOne / 16) <= (uint64_t)(kOne + kOne / 8) && half < kLimit && half > -kLimit;
+    fits &= fits_pair<L>(still, moving, half);
     const int64_t other = __shfl_xor_sync(all, (long long)mine, 16);
     const int64_t x3 = kOne - mine - other;
     fits &= (uint64_t)(x3 + kOne / 16) <= (uint64_t)(kOne + kOne / 8);
@@ -447,7 +470,8 @@ __device__ __forceinline__ bool collide_fixed_lane(double (&f)[L::Q], const Fixe
     const int lane = (int)(threadIdx.x & 31u);
     fits = ((votes >> lane) & (votes >> (lane ^ 16)) & 1u) != 0;
     if (votes == 0) return false;
-    int64_t rest = sum, even = 0;
+    uint64_t rest = (uint64_t)sum;  // modulo 2^64 on the way
+    int64_t even = 0;
     int32_t off = 0;
     double out[Q];
 #pragma unroll
@@ -464,16 +488,16 @@ __device__ __forceinline__ bool collide_fixed_lane(double (&f)[L::Q], const Fixe
         if (ka != 0) {
             const int64_t na = x[ka] - (ds + da);
             out[ka] = to_double(na, e, d);
-            rest -= na;
+            rest -= (uint64_t)na;
             off += d;
         }
         const int64_t nb = x[kb] - (ds - da);
         out[kb] = to_double(nb, e, d);
-        rest -= nb;
+        rest -= (uint64_t)nb;
         off += d;
     }
     int32_t d;
-    out[0] = to_double(rest - off, e, d);
+    out[0] = to_double((int64_t)rest - off, e, d);
     if (fits)
 #pragma unroll
         for (int k = 0; k < Q; ++k) f[k] = out[k];

@@ -247,3 +247,49 @@ def test_range_of_the_diffusivities(lib, pairs, applies):
     D[1, 2] = D[2, 1] = pairs[2]
     f, _ = nodes_of("D2Q5", 2, 4, 0.1, "plain", np.random.default_rng(1))
     assert bool(collide(lib, "D2Q5", 2, f, D, 0)[0]) == applies
+
+
+def wild_nodes(lattice, S, count, g):
+    """Nodes far from equilibrium: moving populations of either sign from 1e-3 to one in
+    magnitude, species by species, with mole fractions in [-1/16, 17/16] (population 0 takes
+    what is left), among them trace species beside a wild one."""
+    Q = len(WEIGHTS[lattice])
+    amp = 10.0 ** g.uniform(-3, 0, (count, S, 1))
+    f = amp * g.uniform(-1.0, 1.0, (count, S, Q))
+    x = g.uniform(-0.05, 1.05, (count, S))
+    f[:, :, 0] = x - f[:, :, 1:].sum(2)
+    calm = np.array(WEIGHTS[lattice]) * x[:, :, None]
+    pick = g.integers(0, 4, count)
+    for s in range(S):
+        f[pick == s, s] = calm[pick == s, s]  # one species at equilibrium
+    trace = pick == 3
+    f[trace, 0] *= 10.0 ** g.uniform(-30, -3, (trace.sum(), 1))
+    if Q in (5, 7, 9, 15):  # opposite pairs that cancel in the sum, one of them large
+        for i in range(0, count, 5):
+            b = g.uniform(0.3, 0.9999)
+            f[i, 0, 1:5] = [b, b, -b, -b]
+            f[i, 0, 5:] *= 0.05
+            f[i, 0, 0] = g.uniform(0.0, 0.9) - f[i, 0, 1:].sum()
+    return f
+
+
+@pytest.mark.parametrize("srt", [0, 1])
+@pytest.mark.parametrize("S", [1, 2])
+@pytest.mark.parametrize("lattice", sorted(WEIGHTS))
+def test_wild_nodes_are_right_or_refused(lib, lattice, S, srt):
+    """Whatever node is taken comes out right to 2^-47 of the species' largest population
+    before or after: the coefficients' errors are at most some 2^-50 of the departures they
+    multiply, for diffusivities within a factor of twelve.  A number that does not fit
+    its field is wrong by orders of magnitude more."""
+    g = np.random.default_rng([7, len(lattice), S, srt, len(WEIGHTS[lattice])])
+    taken = 0
+    for _ in range(4):
+        f = wild_nodes(lattice, S, 20000, g)
+        on, out, err, _, mass, fits = collide(lib, lattice, S, f, matrix(S + 1, g), srt)
+        assert on
+        assert np.array_equal(out[~fits], f[~fits])
+        scale = np.maximum(np.abs(f).max(2), np.abs(out).max(2))
+        assert (np.abs(err[fits]).max(2) <= 2.0 ** -47 * scale[fits]).all()
+        assert (np.abs(mass[fits]) <= 2.0 ** -47 * scale[fits]).all()
+        taken += fits.sum()
+    assert taken > 2000

@@ -69,3 +69,94 @@ def test_steep_fronts_match_the_oracle(n):
         rx, rJ = oracle.run("D2Q5", D, x0, steps, bc=bc, flux=True)
         assert np.abs(x.cpu().numpy() - rx).max() <= 1e-12
         assert np.abs(J.cpu().numpy() - rJ).max() <= 1e-13
+
+
+# Ternary D2Q5 nodes that leave the range of the fixed-point collision (populations of two
+# species: rest, then opposite pairs)
+WILD = {
+    "pair below one": [[0.3, 0.99, 0.99, -0.99, -0.99], [0.1, 0.05, 0.05, 0.05, 0.05]],
+    "pair above a half": [[0.0, 0.55, 0.02, 0.02, 0.02], [0.1, 0.05, 0.05, 0.05, 0.05]],
+    "other species' pair": [[0.1, 0.05, 0.05, 0.05, 0.05], [0.2, -0.97, 0.98, 0.97, -0.96]],
+    "mole fraction 1.2": [[0.4, 0.2, 0.2, 0.2, 0.2], [0.0, 0.01, 0.0, 0.01, 0.0]],
+    "population above one": [[1.5, -0.2, -0.2, -0.2, -0.2], [0.1, 0.05, 0.05, 0.05, 0.05]],
+    "below 2^-900": [[1e-280, 1e-281, 2e-281, 3e-281, 1e-281], [0.1, 0.05, 0.05, 0.05, 0.05]],
+    "third species below zero": [[0.25, 0.1, 0.12, 0.1, 0.12], [0.25, 0.12, 0.1, 0.1, 0.1]],
+}
+
+
+def _collide(f, D):
+    """The D2Q5 collision with Eq. 3-16's even rates of one ternary node, in FP64."""
+    w = np.array([1 / 3] + [1 / 6] * 4)
+    x = f.sum(1)
+    xi = np.append(x, 1.0 - x.sum())
+    B = np.empty((2, 2))
+    for i in range(2):
+        for j in range(2):
+            B[i, j] = (xi[i] * (1 / D[i, 2] - 1 / D[i, j]) if i != j
+                       else xi[i] / D[i, 2] + sum(xi[k] / D[i, k] for k in range(3) if k != i))
+    odd = np.linalg.solve(B / 2 + 3.0 * np.eye(2), B / 2)
+    even = odd.copy()
+    for i in range(2):
+        even[i, i] = 4 * (odd[i, i] - 1) / (odd[i, i] - 4)
+    out = f.copy()
+    for a in (1, 3):
+        s = even @ (f[:, a] + f[:, a + 1] - 2 * w[a] * x)
+        o = odd @ (f[:, a] - f[:, a + 1])
+        out[:, a] -= s + o
+        out[:, a + 1] -= s - o
+    out[:, 0] = x - out[:, 1:].sum(1)
+    return out
+
+
+@pytest.mark.parametrize("grid", [(100, 101), (40, 30), (400, 300)])
+@pytest.mark.parametrize("kind", sorted(WILD))
+def test_wild_nodes_follow_the_fp64_collision(grid, kind):
+    """A uniform periodic field only collides.  Three steps, of two lanes per node, of tiles and
+    of one lane per node by the size of the grid, against the collision in numpy; to
+    2^-47 of the largest population (a few FP64 roundings of departures up to four)."""
+    from paper_1808_06787_gb300 import Solver
+
+    D = sy.random_D(3, seed=4)
+    node = np.array(WILD[kind])
+    s = Solver("D2Q5", D, grid, dtype=torch.float64)
+    f = torch.from_numpy(node)[:, :, None].expand(s.state_shape).contiguous().cuda()
+    s.set_state_raw(f, 0)
+    s.step(3)
+    want = _collide(_collide(_collide(node, D), D), D)
+    got = s.get_state().cpu().numpy()
+    for i in range(2):
+        scale = max(np.abs(node[i]).max(), np.abs(want[i]).max())
+        assert np.abs(got[i] - want[i][:, None]).max() <= 2.0 ** -47 * scale
+
+
+@pytest.mark.parametrize("faces", ["pp", "ww"])
+@pytest.mark.parametrize("grid", [(101, 64), (64, 51)])
+def test_isolated_wild_nodes_take_the_same_path_everywhere(grid, faces):
+    """Single wild nodes in the warps of an ordinary field, the last one among them: a field
+    repeated along a periodic axis until one lane takes a node gives the same populations
+    bit for bit as the field alone (two lanes per node, or tiles)."""
+    from paper_1808_06787_gb300 import Solver
+
+    nx, ny = grid
+    copies = -(-98305 // (nx * ny))
+    bc = ("noflux" if faces == "ww" else "periodic",) * 2 + ("periodic",) * 4
+    D = sy.random_D(3, seed=4)
+    a = Solver("D2Q5", D, (nx, ny), bc=bc, dtype=torch.float64)
+    b = Solver("D2Q5", D, (nx, ny * copies), bc=bc, dtype=torch.float64)
+    g = np.random.default_rng(8)
+    x = g.uniform(0.05, 1.0, (3, nx * ny))
+    x /= x.sum(0)
+    w = np.array([1 / 3] + [1 / 6] * 4)
+    f = w[None, :, None] * x[:2, None, :] * (1 + 0.2 * g.uniform(-1, 1, (2, 5, nx * ny)))
+    at = np.concatenate([[0, 15, 16, 17, nx * ny - 1], g.integers(0, nx * ny, 40)])
+    for i, c in enumerate(at):
+        f[:, :, c] = WILD[sorted(WILD)[i % len(WILD)]]
+    f = torch.from_numpy(f).cuda()
+    a.set_state_raw(f.contiguous(), 0)
+    b.set_state_raw(f.repeat(1, 1, copies).contiguous(), 0)
+    for n in (2, 3, 6):
+        a.step(n)
+        b.step(n)
+        want = a.get_state()
+        assert torch.isfinite(want).all()
+        assert torch.equal(b.get_state(), want.repeat(1, 1, copies))
