@@ -175,6 +175,18 @@ LBMS_HD bool fits_pair(uint32_t rest, uint32_t moving, int64_t half)
     return (int)((rest > moving ? rest : moving) >> 20) <= 1021 && half < kLimit / 2 && half > -kLimit / 2;
 }
 
+// Whether a species' largest exponent field serves as its block exponent; 0 where every
+// population is zero, but not where some are subnormal.
+template <int Q>
+LBMS_HD bool fits_block(int M, const double (&f)[Q])
+{
+    if (M != 0) return M >= 120 && M <= 1022;
+    uint64_t any = 0;
+#pragma unroll
+    for (int k = 0; k < Q; ++k) any |= bits_of(f[k]);
+    return (any << 1) == 0;
+}
+
 LBMS_HD Block block(int M, int bits)
 {
     const int r = 965 + bits - M;
@@ -305,7 +317,7 @@ LBMS_HD bool collide_fixed(double (&f)[S][L::Q], const FixedTable& t)
         }
         const uint32_t top = rest > moving ? rest : moving;
         e[s] = block((int)(top >> 20), block_bits<L>());
-        fits &= e[s].M <= 1022 && (e[s].M == 0 || e[s].M >= 120);
+        fits &= fits_block(e[s].M, f[s]);
         int64_t a = 0;
 #pragma unroll
         for (int k = 0; k < Q; ++k) {
@@ -434,7 +446,7 @@ __device__ __forceinline__ bool collide_fixed_lane(double (&f)[L::Q], const Fixe
     }
     const uint32_t top = still > moving ? still : moving;
     const Block e = block((int)(top >> 20), block_bits<L>());
-    bool fits = active && e.M <= 1022 && (e.M == 0 || e.M >= 120);
+    bool fits = fits_block(e.M, f) && active;
     int64_t x[Q], sum = 0;
 #pragma unroll
     for (int k = 0; k < Q; ++k) {

@@ -293,3 +293,24 @@ def test_wild_nodes_are_right_or_refused(lib, lattice, S, srt):
         assert (np.abs(mass[fits]) <= 2.0 ** -47 * scale[fits]).all()
         taken += fits.sum()
     assert taken > 2000
+
+
+@pytest.mark.parametrize("S", [1, 2])
+@pytest.mark.parametrize("lattice", sorted(WEIGHTS))
+def test_subnormal_species_are_refused(lib, lattice, S):
+    """A species whose populations are all subnormal has a block exponent of zero without
+    being zero: it has to go to the FP64 arithmetic, not to zero."""
+    g = np.random.default_rng(11)
+    f, _ = nodes_of(lattice, S, 8, 0.1, "plain", g)
+    Q = f.shape[2]
+    f[:4, 0] = 0.0
+    f[0, 0] = 5e-324
+    f[1, 0] = -1e-310
+    f[2, 0, Q - 1] = 2e-308
+    f[3, 0, 0] = 1e-320
+    f[4, 0] = 0.0  # exactly absent
+    f[5, 0] = -0.0
+    on, out, _, _, _, fits = collide(lib, lattice, S, f, matrix(S + 1, g), 0)
+    assert on and list(fits) == [False] * 4 + [True] * 4
+    assert np.array_equal(out[:4], f[:4])
+    assert not out[4:6, 0].any()

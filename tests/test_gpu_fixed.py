@@ -80,6 +80,7 @@ WILD = {
     "mole fraction 1.2": [[0.4, 0.2, 0.2, 0.2, 0.2], [0.0, 0.01, 0.0, 0.01, 0.0]],
     "population above one": [[1.5, -0.2, -0.2, -0.2, -0.2], [0.1, 0.05, 0.05, 0.05, 0.05]],
     "below 2^-900": [[1e-280, 1e-281, 2e-281, 3e-281, 1e-281], [0.1, 0.05, 0.05, 0.05, 0.05]],
+    "subnormal species": [[3e-310, 1e-310, 2e-310, 1e-310, 1e-310], [0.1, 0.05, 0.05, 0.05, 0.05]],
     "third species below zero": [[0.25, 0.1, 0.12, 0.1, 0.12], [0.25, 0.12, 0.1, 0.1, 0.1]],
 }
 
@@ -113,7 +114,8 @@ def _collide(f, D):
 def test_wild_nodes_follow_the_fp64_collision(grid, kind):
     """A uniform periodic field only collides.  Three steps, of two lanes per node, of tiles and
     of one lane per node by the size of the grid, against the collision in numpy; to
-    2^-47 of the largest population (a few FP64 roundings of departures up to four)."""
+    2^-47 of the largest population (a few FP64 roundings of departures up to four), or 64
+    subnormal units."""
     from paper_1808_06787_gb300 import Solver
 
     D = sy.random_D(3, seed=4)
@@ -126,7 +128,7 @@ def test_wild_nodes_follow_the_fp64_collision(grid, kind):
     got = s.get_state().cpu().numpy()
     for i in range(2):
         scale = max(np.abs(node[i]).max(), np.abs(want[i]).max())
-        assert np.abs(got[i] - want[i][:, None]).max() <= 2.0 ** -47 * scale
+        assert np.abs(got[i] - want[i][:, None]).max() <= max(2.0 ** -47 * scale, 64 * 5e-324)
 
 
 @pytest.mark.parametrize("faces", ["pp", "ww"])
