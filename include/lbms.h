@@ -187,7 +187,9 @@ int lbms_set_reference(lbms_t* h, const double* xi_ref);
  * The last step of each call also writes per-block partial sums of every
  * species' mole fraction, which lbms_mass reduces when it is called, so
  * lbms_mass after lbms_step reads no populations.  Asynchronous: launch errors are returned at once, numerical
- * trouble is raised in the status flags.  Returns LBMS_EINVAL if a Dirichlet
+ * trouble is raised in the status flags.  While the handle's stream is being captured the
+ * launches go into the caller's graph; a graph of an even number of steps ends in the
+ * buffer it began with, so each launch of it advances that many steps.  Returns LBMS_EINVAL if a Dirichlet
  * face has no composition yet.  With Dirichlet faces the species' masses are
  * not conserved (the faces exchange mass with the outside).
  */
@@ -347,14 +349,15 @@ long lbms_steps_done(const lbms_t* h);
 
 /* Kernel launches that lbms_step(h, n_steps) makes (or replays): grids beyond the
  * L2 cache take several steps per launch on the 1D and 2D lattices in F32, and so do
- * grids too small to fill the chip.  0 for
- * n_steps < 1, -1 for a NULL handle. */
+ * grids too small to fill the chip.  (A call under stream capture may make one more
+ * per 64 steps, see lbms_step.)  0 for n_steps < 1, -1 for a NULL handle. */
 long lbms_step_launches(const lbms_t* h, long n_steps);
 
 /* Device address, inside the caller's workspace, of the buffer that holds the
- * current post-collision populations (layout as lbms_get_state).  It changes
- * with every step (the two buffers alternate) and after lbms_set_state_raw;
- * NULL for a NULL handle. */
+ * current post-collision populations (layout as lbms_get_state).  The two buffers
+ * alternate with every launch of a step kernel (lbms_step_launches: a launch may take
+ * several steps), and lbms_set_state and lbms_set_state_raw choose one, so ask again
+ * after each of these calls and after lbms_step.  NULL for a NULL handle. */
 const void* lbms_populations(const lbms_t* h);
 
 /* Message of the last failed call on this handle ("" if none).  With h == NULL,
@@ -462,7 +465,8 @@ int lbms_batch_set_state(lbms_batch_t* b, const void* x0, const int64_t* offsets
  * (schedule and kernel shape) chosen by lbms_batch_tune or
  * lbms_batch_set_schedule (default: all instances per launch, see below).
  * Each instance evolves exactly as lbms_step would
- * evolve it alone, bit for bit.  The last step writes the mass partials.
+ * evolve it alone, bit for bit.  The last step writes the mass partials.  Under
+ * stream capture as lbms_step.
  */
 int lbms_batch_step(lbms_batch_t* b, long n_steps);
 

@@ -287,8 +287,13 @@ int bdepth(const lbms_batch_t* b)
 }
 
 // Launches a run of n plain steps of the streamed schedule takes (split evenly, as for
-// single solves).
-long bpasses(const lbms_batch_t* b, long n) { return (n + bdepth(b) - 1) / bdepth(b); }
+// single solves).  replay: in a caller's graph their number is even or odd as n is, so that
+// a call of an even number of steps ends in the buffer it began with.
+long bpasses(const lbms_batch_t* b, long n, bool replay = false)
+{
+    const long p = (n + bdepth(b) - 1) / bdepth(b);
+    return replay ? p + ((p ^ n) & 1) : p;
+}
 
 cudaError_t bfinalize(const lbms_batch_t* b, cudaStream_t st)
 {
@@ -344,17 +349,17 @@ int graph_steps(const lbms_batch_t* b)
 }
 
 // Whether launch_body(steps) leaves the state in the other buffer.
-bool run_parity(const lbms_batch_t* b, long steps)
+bool run_parity(const lbms_batch_t* b, long steps, bool replay = false)
 {
-    return ((b->schedule == 0 ? bpasses(b, steps) : steps) & 1) != 0;
+    return ((b->schedule == 0 ? bpasses(b, steps, replay) : steps) & 1) != 0;
 }
 
-cudaError_t launch_body(const lbms_batch_t* b, int parity, int steps, cudaStream_t st)
+cudaError_t launch_body(const lbms_batch_t* b, int parity, int steps, cudaStream_t st, bool replay = false)
 {
     cudaError_t e = cudaSuccess;
     if (b->schedule == 0) {
         int src = parity, left = steps;
-        for (long passes = bpasses(b, steps); passes > 0 && e == cudaSuccess; --passes, src = 1 - src) {
+        for (long passes = bpasses(b, steps, replay); passes > 0 && e == cudaSuccess; --passes, src = 1 - src) {
             const int m = (int)((left + passes - 1) / passes);
             if (m == 1) {
                 e = bstep(b, src, false, 0, b->lay.total_blocks, st);
@@ -659,7 +664,8 @@ int lbms_batch_step(lbms_batch_t* b, long n_steps)
     if (e != cudaSuccess) return bcuda(b, e, "cudaStreamIsCapturing");
     const int gs = graph_steps(b);
     long body = n_steps - 1;
-    if (cs == cudaStreamCaptureStatusNone) {
+    const bool captured = cs != cudaStreamCaptureStatusNone;  // into a caller's graph
+    if (!captured) {
         while (body >= gs) {
             if (!b->graph[b->cur]) {
                 e = build_graph(b, b->cur);
@@ -677,9 +683,9 @@ int lbms_batch_step(lbms_batch_t* b, long n_steps)
     }
     while (body > 0) {
         const int chunk = (int)(body < gs ? body : gs);
-        e = launch_body(b, b->cur, chunk, b->stream);
+        e = launch_body(b, b->cur, chunk, b->stream, captured);
         if (e != cudaSuccess) return bcuda(b, e, "batch step kernel");
-        if (run_parity(b, chunk)) b->cur = 1 - b->cur;
+        if (run_parity(b, chunk, captured)) b->cur = 1 - b->cur;
         body -= chunk;
         b->steps += chunk;
     }

@@ -22,13 +22,15 @@ constexpr size_t kAlign = 256;
 constexpr size_t kStagingMax = size_t(16) << 20;  // host I/O chunk area
 constexpr int kGraphSteps = 32;                   // steps per captured graph (even)
 // captured run lengths: full runs of kGraphSteps, then the even remainder in
-// binary pieces (all even, so a run leaves the buffer parity unchanged)
+// binary pieces (where a launch takes several steps, a piece may be an odd number of
+// launches and leave the state in the other buffer: plain_launches)
 constexpr int kGraphLens[5] = {kGraphSteps, 16, 8, 4, 2};
 // calls of at most kCallGraphMax steps are replayed whole: the plain steps and
 // the mass-writing last one in one graph, kept for the kCallGraphs most
-// recently used (length, parity) pairs
+// recently used (length, parity) pairs; a call of an odd number of launches comes from
+// either parity in turn, so that four lengths may need eight
 constexpr long kCallGraphMax = 64;
-constexpr int kCallGraphs = 4;
+constexpr int kCallGraphs = 8;
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
@@ -401,14 +403,21 @@ cudaError_t launch_fused_steps(const lbms_t* h, int src, int m, cudaStream_t st)
     return dispatch_tile(h->lattice, h->dtype, a);
 }
 
-// Launches a run of n plain steps takes: passes of at most h->depth steps.
-long plain_launches(const lbms_t* h, long n) { return (n + h->depth - 1) / h->depth; }
+// Launches a run of n plain steps takes: passes of at most h->depth steps.  Every launch
+// changes buffers.  replay: a caller's graph may be launched again from the buffer it began
+// with, so that a call of an even number of steps has to end there, as single steps do;
+// one pass more then where the parities differ.
+long plain_launches(const lbms_t* h, long n, bool replay = false)
+{
+    const long p = (n + h->depth - 1) / h->depth;
+    return replay ? p + ((p ^ n) & 1) : p;
+}
 
 // n plain steps from f[src], split evenly over the passes (so that none is left a
 // single step where it can be helped); src becomes the buffer that holds the result.
-cudaError_t launch_plain(const lbms_t* h, int& src, long n, cudaStream_t st)
+cudaError_t launch_plain(const lbms_t* h, int& src, long n, cudaStream_t st, bool replay = false)
 {
-    for (long passes = plain_launches(h, n); passes > 0; --passes) {
+    for (long passes = plain_launches(h, n, replay); passes > 0; --passes) {
         const int m = (int)((n + passes - 1) / passes);
         cudaError_t e = m == 1 ? launch_step(h, src, false, st) : launch_fused_steps(h, src, m, st);
         if (e != cudaSuccess) return e;
@@ -871,7 +880,8 @@ int lbms_step(lbms_t* h, long n_steps)
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(h->stream, &cs);
     if (e != cudaSuccess) return cuda_fail(h, e, "cudaStreamIsCapturing");
-    const bool use_graphs = h->graphs_ok && cs == cudaStreamCaptureStatusNone;
+    const bool captured = cs != cudaStreamCaptureStatusNone;  // into a caller's graph
+    const bool use_graphs = h->graphs_ok && !captured;
     if (use_graphs && n_steps >= 2 && n_steps <= kCallGraphMax) {
         cudaGraphExec_t g = call_graph_for(h, n_steps);
         if (g) {
@@ -906,7 +916,7 @@ int lbms_step(lbms_t* h, long n_steps)
     }
     while (left > 1) {
         const long m = left - 1 < kCallGraphMax ? left - 1 : kCallGraphMax;
-        e = launch_plain(h, h->cur, m, h->stream);
+        e = launch_plain(h, h->cur, m, h->stream, captured);
         if (e != cudaSuccess) return cuda_fail(h, e, "step kernel");
         left -= m;
         h->steps += m;
