@@ -340,13 +340,17 @@ __device__ __forceinline__ uint32_t grid_block(int reverse)
 // Blocks per SM the FP32 step kernels are compiled for (register budget): one
 // node per thread keeps S * Q populations and the S x S matrices in registers,
 // and enough resident warps must remain to cover HBM latency.  FP64 binary and ternary
-// steps (fixed.cuh) at 3 blocks: D2Q5 1024^2 66.4 / 66.4 / 55 us per step at 1 / 2 / 3, D3Q7
-// 101 x 96 x 67 50.7 / 50.7 / 46 (four alike, but D2Q9 300^2 12.6 -> 15.9).
+// steps (fixed.cuh) at 3 blocks of 80 registers while a thread holds up to 18 populations: us
+// per step at 1 / 2 / 3, D2Q5 1024^2 66.4 / 66.4 / 55, D3Q7 101 x 96 x 67 50.7 / 50.7 / 46 (four
+// alike, but D2Q9 300^2 12.6 -> 15.9), D2Q9 1024^2 94 / 93 / 94 (mass-writing 154 / 151 / 154).
+// The 30 of D3Q15's ternary nodes spill 776 bytes there and take 2 blocks: 128^3 386 / 309 /
+// 364 (mass-writing 604 / 484 / 498), 64^3 51 / 43 / 52, in FP64 arithmetic (frozen)
+// 1220 / 1110 / 1220; its binary nodes keep 3 (129 / 129 / 114).
 template <int LAT, int S, typename T>
 struct StepOccupancy {
     static constexpr int P = S * Lattice<LAT>::Q;  // populations held per thread
     static constexpr int value =
-        sizeof(T) != 4 ? (S <= 2 ? 3 : 1)
+        sizeof(T) != 4 ? (S > 2 ? 1 : (P <= 18 ? 3 : 2))
         : Lattice<LAT>::Q <= 9 ? (S <= 2 ? 6 : (S == 3 ? 4 : (S == 4 ? 3 : 2)))
                                : (P <= 15 ? 4 : (P <= 30 ? 3 : 2));
 };
