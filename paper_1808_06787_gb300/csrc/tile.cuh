@@ -105,8 +105,12 @@ cudaError_t launch_tile(const KArgs& a)
     const Tiles& t = a.tiles;
     const int region = t.rx * t.ry * t.rz;
     const size_t shared = (size_t)(t.depth > 2 ? 2 : 1) * region * S * Lattice<LAT>::Q * sizeof(T);
+    // The limit belongs to the kernel, not to a launch, and other threads launch it too: every
+    // one of them sets the same, the most a pass of it can take.
+    constexpr size_t most = size_t(2) * kTileThreads * S * Lattice<LAT>::Q * sizeof(T);
+    static_assert(most <= size_t(227) << 10, "more than a block has");
     if (shared > size_t(48) << 10) {
-        cudaError_t e = cudaFuncSetAttribute(k_step_tile<LAT, S, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shared);
+        cudaError_t e = cudaFuncSetAttribute(k_step_tile<LAT, S, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
         if (e != cudaSuccess) return e;
     }
     const uint32_t blocks = (uint32_t)t.nx * (uint32_t)t.ny * (uint32_t)((a.nz + t.tz - 1) / t.tz);
