@@ -1,4 +1,4 @@
-// Tiled passes of the D2Q9 lattice (two to four species, float and double).
+// Tiled passes of the D2Q9 lattice (two to four species in float, two and three in double).
 #include "tile.cuh"
 
 namespace lbms {

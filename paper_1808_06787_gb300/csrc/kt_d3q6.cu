@@ -1,4 +1,4 @@
-// Tiled passes of the D3Q6 lattice (two to four species, float and double).
+// Tiled passes of the D3Q6 lattice (two and three species, float).
 #include "tile.cuh"
 
 namespace lbms {
@@ -6,7 +6,7 @@ namespace lbms {
 template <>
 cudaError_t dispatch_tile_lattice<LBMS_D3Q6>(int dtype, const KArgs& a)
 {
-    return dtype == LBMS_F64 ? launch_tile_species<LBMS_D3Q6, double>(a) : launch_tile_species<LBMS_D3Q6, float>(a);
+    return dtype == LBMS_F64 ? cudaErrorInvalidValue : launch_tile_species<LBMS_D3Q6, float>(a);
 }
 
 }  // namespace lbms

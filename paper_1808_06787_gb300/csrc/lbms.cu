@@ -13,6 +13,7 @@
 #include "adjoint.cuh"
 #include "lbms_internal.h"
 #include "node.cuh"
+#include "plan.h"
 
 using namespace lbms;
 
@@ -221,7 +222,7 @@ struct lbms_s {
     uint32_t cells = 0, blocks = 0;  // blocks: of the step and mass kernels (mass partial slots)
     uint32_t step_block = 256;        // their threads per block
     int sms = 1;                      // multiprocessors of the device
-    int depth = 1;                    // most plain steps one launch takes (fused_depth, tile_depth)
+    int depth = 1;                    // most plain steps one launch takes (tile_shape, fused_depth)
     int tile[3] = {0, 0, 0};          // nodes of a tile, where the passes are tiled
     uint32_t noflux = 0;
     uint32_t dirichlet = 0;  // Dirichlet faces
@@ -458,49 +459,6 @@ int fused_depth(const lbms_t* h)
     return fused_limit_of(h->lattice, h->n);
 }
 
-// Most steps a tiled pass takes (tile.cuh), and its tile; 1 where single steps are faster:
-// above these sizes the margins, formed by several blocks, cost more than the waits they
-// save.  Times, us per step, single -> tiled: FP32 D2Q5 ternary 48 x 40 1.73 ->
-// 0.77, 128^2 1.77 -> 0.91, 200^2 2.03 -> 1.61, 256^2 2.09 -> 1.88, D2Q9 128^2 2.01 -> 1.16,
-// four species 128^2 1.95 -> 1.15 and 200^2 2.23 -> 2.16, binary 256^2 2.13 -> 1.24; D3Q7
-// 24 x 16 x 12 1.79 -> 1.33, 28 x 24 x 16 1.95 -> 1.63, 40 x 24 x 24 2.08 -> 2.10 (single);
-// FP64 binary 240 x 40 1.79 -> 1.22, 128^2 1.78 -> 1.44, 180^2 2.04 -> 2.10 (single),
-// ternary 64^2 2.84 -> 2.43, 80^2 2.98 -> 2.68, 100^2 2.97 -> 3.25 (single), D2Q9 64^2 4.67 ->
-// 3.96; D1Q3 lines of 100 to 8000 nodes FP64 2.4 -> 1.65, FP32 four species 1.59 -> 0.58,
-// 30000 nodes FP64 3.08 -> 3.96 (single).
-int tile_depth(const lbms_t* h, int (&tile)[3])
-{
-    tile[0] = tile[1] = tile[2] = 0;
-    if (h->halo || h->S > 3 || h->lattice == LBMS_D3Q15) return 1;
-    const uint32_t n = h->cells;
-    int K = 1;
-    auto take = [&](int depth, int x, int y, int z) {
-        K = depth;
-        tile[0] = x;
-        tile[1] = y;
-        tile[2] = z;
-    };
-    if (h->dim == 1) {
-        if (n <= 8192 && (h->dtype == LBMS_F32 || h->S <= 2)) take(8, 16, 1, 1);
-    } else if (h->dim == 3) {
-        if (h->dtype == LBMS_F32 && h->S <= 2) {
-            if (n <= 7168) take(3, 4, 4, 4);
-            else if (n <= 12288) take(2, 8, 4, 4);
-        }
-    } else if (h->dtype == LBMS_F32) {
-        if (n <= 8192) take(5, 8, 8, 1);
-        else if (n <= 24576) take(4, 16, 8, 1);
-        else if (n <= 65536) take(h->S == 2 && h->Q <= 5 && n > 40960 ? 2 : 3, 16, 16, 1);
-    } else if (h->S == 1) {
-        if (n <= 9728) take(5, 8, 8, 1);
-        else if (n <= 20480) take(4, 16, 8, 1);
-    } else if (h->S == 2) {
-        if (n <= 4096) take(4, 8, 4, 1);
-        else if (n <= 6400) take(5, 8, 8, 1);
-    }
-    return K;
-}
-
 // The captured graphs hold the kernel arguments: dropped whenever those change.
 void drop_graphs(lbms_t* h)
 {
@@ -729,11 +687,17 @@ int lbms_create(lbms_t** out, int lattice, int n_species, const int grid[3], con
     h->halo = halo;
     h->plane = (uint32_t)split_plane(lattice, grid);
     h->es = dtype == LBMS_F64 ? 8 : 4;
-    h->depth = tile_depth(h, h->tile);
-    if (h->depth == 1) h->depth = fused_depth(h);
     for (int i = 0; i < n; ++i)
         for (int j = 0; j < n; ++j) h->invD[i][j] = i == j ? 0.0 : 1.0 / D[i * n + j];
     if (dtype == LBMS_F64) h->fixed = fixed_table(n, h->invD, lattice_cs2(lattice), relax);
+    if (!halo) {
+        const TileShape t = tile_shape(dim, h->Q, h->S, dtype == LBMS_F64, h->fixed.on != 0, h->nx, h->ny, h->nz, sms);
+        h->depth = t.depth;
+        h->tile[0] = t.x;
+        h->tile[1] = t.y;
+        h->tile[2] = t.z;
+    }
+    if (h->depth == 1) h->depth = fused_depth(h);
     h->ws = static_cast<char*>(workspace);
     h->lay = L;
     h->f[0] = h->ws + L.off_f0;

@@ -124,7 +124,8 @@ cudaError_t launch_tile_species(const KArgs& a)
     switch (a.n_species) {
         case 2: return launch_tile<LAT, 1, T>(a);
         case 3: return launch_tile<LAT, 2, T>(a);
-        case 4: return launch_tile<LAT, 3, T>(a);
+        case 4:
+            if constexpr (sizeof(T) == 4 && Lattice<LAT>::DIM < 3) return launch_tile<LAT, 3, T>(a);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -1,0 +1,97 @@
+"""The rules that choose passes of several steps (plan.h), compiled for the host.
+
+Tiles: whatever the grid's shape, a launch forms a bounded number of nodes per
+multiprocessor and step; a grid of few nodes but many tiles (one node wide, or flat) takes
+single steps.
+"""
+
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+SMS = 152
+
+SOURCE = r"""
+#include "plan.h"
+extern "C" int tiles(int dim, int q, int s, int f64, int fixed, int nx, int ny, int nz, int sms, int* out)
+{
+    const lbms::TileShape t = lbms::tile_shape(dim, q, s, f64 != 0, fixed != 0, nx, ny, nz, sms);
+    out[0] = t.x; out[1] = t.y; out[2] = t.z;
+    return t.depth;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    d = tmp_path_factory.mktemp("plan")
+    src, so = str(d / "plan.cpp"), str(d / "plan.so")
+    with open(src, "w") as f:
+        f.write(SOURCE)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-Wall", "-Werror", "-shared", "-fPIC",
+                    "-I", os.path.join(ROOT, "paper_1808_06787_gb300", "csrc"), src, "-o", so], check=True)
+    return ctypes.CDLL(so)
+
+
+def tile(lib, dim, q, s, f64, fixed, grid):
+    out = (ctypes.c_int * 3)()
+    g = tuple(grid) + (1,) * (3 - len(grid))
+    return lib.tiles(dim, q, s, f64, fixed, *g, SMS, out), tuple(out)
+
+
+KINDS = [(1, 3), (2, 4), (2, 5), (2, 9), (3, 6), (3, 7), (3, 15)]
+
+
+def grids(dim, g):
+    shapes = [(1,) * dim, (8192,) + (1,) * (dim - 1), (1,) * (dim - 1) + (8192,), (65536,) + (1,) * (dim - 1)]
+    for _ in range(600):
+        cells = np.exp(g.uniform(0, np.log(200000)))
+        e = g.dirichlet((0.7,) * dim)
+        shapes.append(tuple(max(1, int(cells ** v)) for v in e))
+    return shapes + [(2 ** 31 - 1,) + (1,) * (dim - 1)]
+
+
+@pytest.mark.parametrize("f64,fixed", [(0, 0), (1, 1), (1, 0)])
+@pytest.mark.parametrize("s", [1, 2, 3, 4, 7])
+@pytest.mark.parametrize("dim,q", KINDS)
+def test_tiles_form_a_bounded_number_of_nodes(lib, dim, q, s, f64, fixed):
+    g = np.random.default_rng([dim, q, s, f64, fixed])
+    taken = 0
+    for grid in grids(dim, g):
+        depth, size = tile(lib, dim, q, s, f64, fixed, grid)
+        assert 1 <= depth <= 8
+        if depth == 1:
+            assert size == (0, 0, 0)
+            continue
+        taken += 1
+        count = np.prod([-(-n // t) for n, t in zip(grid, size)])
+        region = np.prod([t + 2 * (depth - 1) for t in size[:dim]])
+        assert region <= 512 and all(t == 1 for t in size[dim:])
+        # per multiprocessor 1.8 tiles of 400 nodes (FP32) or 1.1 of 308 (FP64); lines 3.4 of 30
+        bound = 3.375 * 30 if dim == 1 else (1.1 * 308 if f64 else 1.8 * 400)
+        assert count * region <= bound * SMS, (grid, depth, size)
+        if s == 3 and size[0] == 16 and size[1] == 16:
+            assert count <= SMS
+        if f64 and not fixed and dim > 1:
+            assert depth == 2 and count <= SMS
+    assert (taken > 20) == (s <= 3 and not (f64 and s > 2) and (dim < 3 or (q < 15 and s <= 2 and not f64)))
+
+
+def test_ordinary_grids_keep_their_tiles(lib):
+    assert tile(lib, 2, 5, 2, 0, 0, (48, 40)) == (5, (8, 8, 1))
+    assert tile(lib, 2, 5, 2, 0, 0, (128, 128)) == (4, (16, 8, 1))
+    assert tile(lib, 2, 9, 2, 0, 0, (256, 256)) == (3, (16, 16, 1))
+    assert tile(lib, 2, 5, 2, 0, 0, (256, 256)) == (2, (16, 16, 1))
+    assert tile(lib, 2, 5, 1, 1, 1, (240, 40)) == (5, (8, 8, 1))
+    assert tile(lib, 2, 5, 2, 1, 1, (64, 64)) == (4, (8, 4, 1))
+    assert tile(lib, 2, 5, 2, 1, 1, (128, 128))[0] == 1
+    assert tile(lib, 3, 7, 2, 0, 0, (24, 16, 12)) == (3, (4, 4, 4))
+    for grid in ((65536, 1), (1, 65536), (24576, 1), (2, 32768)):
+        assert tile(lib, 2, 5, 2, 0, 0, grid)[0] == 1
+    assert tile(lib, 3, 7, 2, 0, 0, (7168, 1, 1))[0] == 1
+    assert tile(lib, 2, 5, 2, 1, 1, (6400, 1))[0] == 1
