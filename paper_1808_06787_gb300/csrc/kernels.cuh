@@ -19,8 +19,9 @@ struct FixedArg<double> {
     FixedTable table;
 };
 
-// Collision of one FP64 node in fixed point (fixed.cuh), for binary and ternary mixtures;
-// false where the FP64 arithmetic has to take it.
+// Collision of one FP64 node in fixed point (fixed.cuh) where its mixture has the
+// coefficients for it (batches, whose instances differ); false where the FP64 arithmetic has
+// to take it.
 template <int LAT, int S>
 __device__ __forceinline__ bool try_fixed(double (&f)[S][Lattice<LAT>::Q], const FixedTable& t)
 {
@@ -29,12 +30,6 @@ __device__ __forceinline__ bool try_fixed(double (&f)[S][Lattice<LAT>::Q], const
     }
     return false;
 }
-template <int LAT, int S, typename Any>
-__device__ __forceinline__ bool try_fixed(float (&)[S][Lattice<LAT>::Q], const Any&)
-{
-    return false;
-}
-
 template <typename T>
 struct Coeffs {
     T invD[LBMS_MAX_SPECIES][LBMS_MAX_SPECIES];  // 1/D_ij times make_coeffs' scale
@@ -87,10 +82,12 @@ struct StepParams {
 // visible (a wait the hardware resolves, not a spin on memory), then lets the
 // following grid be scheduled.  Arithmetic on the launch parameters alone may
 // come first.  In a grid launched without the attribute both return at once.
+__device__ __forceinline__ void await_previous_grid_only() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void admit_next_grid() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void await_previous_grid()
 {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    await_previous_grid_only();
+    admit_next_grid();
 }
 
 // Launches `kernel` with programmatic stream serialisation: only the
@@ -344,13 +341,13 @@ __device__ __forceinline__ uint32_t grid_block(int reverse)
 // per step at 1 / 2 / 3, D2Q5 1024^2 66.4 / 66.4 / 55, D3Q7 101 x 96 x 67 50.7 / 50.7 / 46 (four
 // alike, but D2Q9 300^2 12.6 -> 15.9), D2Q9 1024^2 94 / 93 / 94 (mass-writing 154 / 151 / 154).
 // The 30 of D3Q15's ternary nodes spill 776 bytes there and take 2 blocks: 128^3 386 / 309 /
-// 364 (mass-writing 604 / 484 / 498), 64^3 51 / 43 / 52, in FP64 arithmetic (frozen)
-// 1220 / 1110 / 1220; its binary nodes keep 3 (129 / 129 / 114).
-template <int LAT, int S, typename T>
+// 364 (mass-writing 604 / 484 / 498), 64^3 51 / 43 / 52; its binary nodes keep 3
+// (129 / 129 / 114).
+template <int LAT, int S, typename T, bool FIXED>
 struct StepOccupancy {
     static constexpr int P = S * Lattice<LAT>::Q;  // populations held per thread
     static constexpr int value =
-        sizeof(T) != 4 ? (S > 2 ? 1 : (P <= 18 ? 3 : 2))
+        sizeof(T) != 4 ? (!FIXED ? 1 : (P <= 18 ? 3 : 2))
         : Lattice<LAT>::Q <= 9 ? (S <= 2 ? 6 : (S == 3 ? 4 : (S == 4 ? 3 : 2)))
                                : (P <= 15 ? 4 : (P <= 30 ? 3 : 2));
 };
@@ -359,13 +356,21 @@ struct StepOccupancy {
 // fractions (Eq. 3-15), relaxation matrices (Eqs. 2-10, 3-26, 3-16), collision
 // (Eq. 3-13a with f_eq of Eq. 3-3) and store of the post-collision populations.
 // HALO: the grid is a slab with cut faces (slab decomposition); kernels of
-// undivided grids are compiled without the halo code.
-template <int LAT, int S, typename T, bool MASS, bool HALO>
-__global__ void __launch_bounds__(kBlock, StepOccupancy<LAT, S, T>::value) k_step(StepParams<T> p)
+// undivided grids are compiled without the halo code.  FIXED: the collision runs in fixed
+// point (FP64, fixed.cuh); solvers it does not apply to have kernels without it, for its
+// code and its register budget cost them (us per step, with it -> without: binary D2Q9 128^2
+// 6.9 -> 4.5, 300^2 24.5 -> 19.2).  These are bound by the FP64 pipe of the busiest SM, so
+// they let the next grid in only when they are about to store: blocks that wait beside
+// running ones gather on the SMs that were done first (binary D2Q5 128^2 4.5 -> 3.3, 400^2
+// 27.8 -> 19.5, ternary 300^2 33.1 -> 25.9, D1Q3 of 98000 nodes 28.1 -> 18.3).
+template <int LAT, int S, typename T, bool MASS, bool HALO, bool FIXED = false>
+__global__ void __launch_bounds__(kBlock, StepOccupancy<LAT, S, T, FIXED>::value) k_step(StepParams<T> p)
 {
     using L = Lattice<LAT>;
     constexpr int Q = L::Q;
-    await_previous_grid();
+    constexpr bool kLate = S <= 2 && sizeof(T) == 8 && !FIXED;
+    if constexpr (kLate) await_previous_grid_only();
+    else await_previous_grid();
     const uint32_t lb = grid_block(p.reverse);
     const uint32_t cell = lb * blockDim.x + threadIdx.x;
     const bool active = cell < p.g.cells;
@@ -377,11 +382,11 @@ __global__ void __launch_bounds__(kBlock, StepOccupancy<LAT, S, T>::value) k_ste
         T f[S][Q];
         pull<LAT, S, T>(p.fin, p.g, cell, h, f, p.xb, HALO ? &p.halo : nullptr);
         bool done = false;
-        if constexpr (sizeof(T) == 4 || MASS) mole_fractions<LAT, S, T>(f, xi);
+        if constexpr (!FIXED || MASS) mole_fractions<LAT, S, T>(f, xi);
         if (MASS) check_range<S, T>(xi, p.status);  // once per lbms_step call
-        if constexpr (sizeof(T) == 8) done = try_fixed<LAT, S>(f, p.fixed.table);
+        if constexpr (FIXED) done = collide_fixed<L, S>(f, p.fixed.table);
         if (!done) {
-            if constexpr (sizeof(T) == 8 && !MASS) mole_fractions<LAT, S, T>(f, xi);
+            if constexpr (FIXED && !MASS) mole_fractions<LAT, S, T>(f, xi);
             T L1[S][S], L2[S][S];
             T xl[S + 1];
             lambda_composition<S, T>(xi, p.co, p.relax, xl);
@@ -391,6 +396,7 @@ __global__ void __launch_bounds__(kBlock, StepOccupancy<LAT, S, T>::value) k_ste
             collide<LAT, S, T>(f, xi, L1, L2,
                                mix32(step * 0x9e3779b9u) ^ ((HALO ? cell + p.g.origin : cell) * 0x27d4eb2du));
         }
+        if constexpr (kLate) admit_next_grid();
 #pragma unroll
         for (int s = 0; s < S; ++s)
 #pragma unroll
@@ -860,9 +866,11 @@ cudaError_t launch(Op op, const KArgs& a)
         if constexpr (HALO_STEPS) {
             // slabs step one exchange at a time: every step writes the mass
             // partials (one kernel variant instead of two)
-            if (op == OP_STEP || op == OP_STEP_MASS)
-                return launch_chained(k_step<LAT, S, T, true, true>, blocks, tb, a.stream, p);
-            return cudaErrorInvalidValue;
+            if (op != OP_STEP && op != OP_STEP_MASS) return cudaErrorInvalidValue;
+            if constexpr (S <= 2 && sizeof(T) == 8) {
+                if (a.fixed.on) return launch_chained(k_step<LAT, S, T, true, true, true>, blocks, tb, a.stream, p);
+            }
+            return launch_chained(k_step<LAT, S, T, true, true>, blocks, tb, a.stream, p);
         } else {
             if constexpr (pair_kernel_lattice<LAT, S, T>()) {
                 // grids whose state stays in L2 keep one node per thread (more
@@ -878,6 +886,12 @@ cudaError_t launch(Op op, const KArgs& a)
                 if (op == OP_STEP && a.fixed.on && a.cells <= kSpeciesMaxCells)
                     return launch_chained(k_step_species<LAT>, (a.cells + kSmallBlock / 2 - 1) / (kSmallBlock / 2),
                                           kSmallBlock, a.stream, p);
+            }
+            if constexpr (S <= 2 && sizeof(T) == 8) {
+                if (op == OP_STEP && a.fixed.on)
+                    return launch_chained(k_step<LAT, S, T, false, false, true>, blocks, tb, a.stream, p);
+                if (op == OP_STEP_MASS && a.fixed.on)
+                    return launch_chained(k_step<LAT, S, T, true, false, true>, blocks, tb, a.stream, p);
             }
             if (op == OP_STEP) return launch_chained(k_step<LAT, S, T, false, false>, blocks, tb, a.stream, p);
             if (op == OP_STEP_MASS) return launch_chained(k_step<LAT, S, T, true, false>, blocks, tb, a.stream, p);

@@ -15,13 +15,13 @@
 
 namespace lbms {
 
-// Collision of one node, in fixed point where that applies (k_step's arithmetic).
-template <int LAT, int S, typename T>
+// Collision of one node (k_step's arithmetic; FIXED as there).
+template <int LAT, int S, typename T, bool FIXED>
 __device__ __forceinline__ void advance_node(T (&f)[S][Lattice<LAT>::Q], const StepParams<T>& p, uint32_t key)
 {
     using L = Lattice<LAT>;
-    if constexpr (sizeof(T) == 8) {
-        if (try_fixed<LAT, S>(f, p.fixed.table)) return;
+    if constexpr (FIXED) {
+        if (collide_fixed<L, S>(f, p.fixed.table)) return;
     }
     T xi[S + 1], xl[S + 1], L1[S][S], L2[S][S];
     mole_fractions<LAT, S, T>(f, xi);
@@ -30,7 +30,7 @@ __device__ __forceinline__ void advance_node(T (&f)[S][Lattice<LAT>::Q], const S
     collide<LAT, S, T>(f, xi, L1, L2, key);
 }
 
-template <int LAT, int S, typename T>
+template <int LAT, int S, typename T, bool FIXED>
 __global__ void __launch_bounds__(kTileThreads) k_step_tile(StepParams<T> p, Tiles t)
 {
     using L = Lattice<LAT>;
@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(kTileThreads) k_step_tile(StepParams<T> p, Til
     T f[S][Q];
     if (inside) {
         pull<LAT, S, T>(p.fin, p.g, cell, h, f, p.xb);
-        advance_node<LAT, S, T>(f, p, mix32(step * 0x9e3779b9u) ^ (cell * 0x27d4eb2du));
+        advance_node<LAT, S, T, FIXED>(f, p, mix32(step * 0x9e3779b9u) ^ (cell * 0x27d4eb2du));
     }
     // within the region neighbours lie next to each other whatever the grid's wraps
     h.ox[0] = -1;
@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(kTileThreads) k_step_tile(StepParams<T> p, Til
         __syncthreads();
         if (inside && edge >= l) {
             pull<LAT, S, T>(now, g, (uint32_t)i, h, f, p.xb);
-            advance_node<LAT, S, T>(f, p, mix32((step + l) * 0x9e3779b9u) ^ (cell * 0x27d4eb2du));
+            advance_node<LAT, S, T, FIXED>(f, p, mix32((step + l) * 0x9e3779b9u) ^ (cell * 0x27d4eb2du));
         }
     }
     // the tile's own nodes (those beyond a ragged end belong to nobody, or wrapped to others)
@@ -99,8 +99,8 @@ __global__ void __launch_bounds__(kTileThreads) k_step_tile(StepParams<T> p, Til
     }
 }
 
-template <int LAT, int S, typename T>
-cudaError_t launch_tile(const KArgs& a)
+template <int LAT, int S, typename T, bool FIXED>
+cudaError_t launch_tile_of(const KArgs& a)
 {
     const Tiles& t = a.tiles;
     const int region = t.rx * t.ry * t.rz;
@@ -110,12 +110,21 @@ cudaError_t launch_tile(const KArgs& a)
     constexpr size_t most = size_t(2) * kTileThreads * S * Lattice<LAT>::Q * sizeof(T);
     static_assert(most <= size_t(227) << 10, "more than a block has");
     if (shared > size_t(48) << 10) {
-        cudaError_t e = cudaFuncSetAttribute(k_step_tile<LAT, S, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+        cudaError_t e = cudaFuncSetAttribute(k_step_tile<LAT, S, T, FIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
         if (e != cudaSuccess) return e;
     }
     const uint32_t blocks = (uint32_t)t.nx * (uint32_t)t.ny * (uint32_t)((a.nz + t.tz - 1) / t.tz);
-    return launch_chained_shared(k_step_tile<LAT, S, T>, blocks, (uint32_t)(region + 31) / 32 * 32, shared, a.stream,
+    return launch_chained_shared(k_step_tile<LAT, S, T, FIXED>, blocks, (uint32_t)(region + 31) / 32 * 32, shared, a.stream,
                                  make_step_params<T>(a), t);
+}
+
+template <int LAT, int S, typename T>
+cudaError_t launch_tile(const KArgs& a)
+{
+    if constexpr (sizeof(T) == 8) {
+        if (a.fixed.on) return launch_tile_of<LAT, S, T, true>(a);
+    }
+    return launch_tile_of<LAT, S, T, false>(a);
 }
 
 template <int LAT, typename T>
