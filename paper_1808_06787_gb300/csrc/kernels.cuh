@@ -336,8 +336,12 @@ __device__ __forceinline__ uint32_t grid_block(int reverse)
 
 // Blocks per SM the FP32 step kernels are compiled for (register budget): one
 // node per thread keeps S * Q populations and the S x S matrices in registers,
-// and enough resident warps must remain to cover HBM latency.  FP64 binary and ternary
-// steps (fixed.cuh) at 3 blocks of 80 registers while a thread holds up to 18 populations: us
+// and enough resident warps must remain to cover HBM latency.  Four species on D2Q4 and
+// D2Q5 at 5 blocks (us per step at 4 / 5: D2Q5 300^2 4.04 / 3.32, 700^2 9.54 / 9.32), five on D3Q6
+// at 4 (40^3 4.65 / 3.44, 100^3 34.2 / 33.2 at 3 / 4): the blocks of two steps then fit side by
+// side where a step has two or three per SM.
+// FP64 binary and ternary steps (fixed.cuh) at 3 blocks of 80 registers while a thread
+// holds up to 18 populations: us
 // per step at 1 / 2 / 3, D2Q5 1024^2 66.4 / 66.4 / 55, D3Q7 101 x 96 x 67 50.7 / 50.7 / 46 (four
 // alike, but D2Q9 300^2 12.6 -> 15.9), D2Q9 1024^2 94 / 93 / 94 (mass-writing 154 / 151 / 154).
 // The 30 of D3Q15's ternary nodes spill 776 bytes there and take 2 blocks: 128^3 386 / 309 /
@@ -348,7 +352,8 @@ struct StepOccupancy {
     static constexpr int P = S * Lattice<LAT>::Q;  // populations held per thread
     static constexpr int value =
         sizeof(T) != 4 ? (!FIXED ? 1 : (P <= 18 ? 3 : 2))
-        : Lattice<LAT>::Q <= 9 ? (S <= 2 ? 6 : (S == 3 ? 4 : (S == 4 ? 3 : 2)))
+        : Lattice<LAT>::Q <= 9 ? (S <= 2 ? 6 : S == 3 ? (Lattice<LAT>::Q <= 5 ? 5 : 4)
+                                          : S == 4 ? (Lattice<LAT>::Q == 6 ? 4 : 3) : 2)
                                : (P <= 15 ? 4 : (P <= 30 ? 3 : 2));
 };
 

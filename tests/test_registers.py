@@ -38,3 +38,17 @@ def test_fp64_steps_spill_no_more_than_their_populations(lat, s, fixed, tmp_path
     assert r.returncode == 0, r.stderr
     spills = [int(v) for v in re.findall(r"(\d+) bytes spill stores", r.stderr)]
     assert len(spills) >= 2 and max(spills) <= (2 * 8 * s * int(lat[8:]) if fixed == "true" else 0), spills
+
+
+@pytest.mark.parametrize("lat,s,most", [("LBMS_D2Q5", 3, 48), ("LBMS_D2Q4", 3, 48), ("LBMS_D3Q6", 4, 64)])
+def test_fp32_steps_leave_room_for_the_next_grid(lat, s, most, tmp_path):
+    """Blocks of 256 threads: five per SM with 48 registers, four with 64."""
+    src = tmp_path / "k.cu"
+    src.write_text('#include "kernels.cuh"\nnamespace lbms {\n'
+                   "template __global__ void k_step<%s, %d, float, false, false>(StepParams<float>);\n}\n" % (lat, s))
+    r = subprocess.run([build.nvcc()] + build.ARCH + build.NVCC_FLAGS
+                       + ["-Xptxas", "-v", "-c", str(src), "-o", os.devnull],
+                       capture_output=True, text=True, cwd=str(tmp_path))
+    assert r.returncode == 0, r.stderr
+    used = [int(v) for v in re.findall(r"Used (\d+) registers", r.stderr)]
+    assert used and max(used) <= most, used
