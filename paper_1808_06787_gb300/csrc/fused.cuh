@@ -21,6 +21,7 @@
 #include <type_traits>
 
 #include "kernels.cuh"
+#include "plan.h"
 
 namespace lbms {
 
@@ -85,13 +86,8 @@ struct March {
 
 constexpr int kFusedBlock = 128;
 
-// Rows of a plane (2D).  A lane owns one column of its warp's strip of 32 columns,
-// K - 1 of them on each side only to feed the later steps.
-template <int K>
-struct Strip {
-    static constexpr int H = K - 1;
-    static constexpr int W = 32 - 2 * H;
-};
+// Rows of a plane (2D).  A lane owns one column of its warp's strip of 32 columns, K - 1 of
+// them on each side only to feed the later steps (row_plan, plan.h).
 
 // The grid a warp marches through: a plane of its own, or one of a batch's (whose nodes
 // begin at `base` of a common node space).
@@ -209,17 +205,9 @@ struct RowQueue {
     }
 };
 
-// Blocks of 4 warps per SM the row kernels are compiled for.  What bounds them is the
-// issue rate (D2Q5 ternary: 216 instructions per 32 nodes and step, of them 122 FP32, at
-// 0.75 per clock; HBM runs at 2.8 TB/s of its 6.8), so each value is the fewest warps
-// that still keep issuing, with the registers that leaves.  Measured, us per step, at
-// blocks 2 / 3 / 4 / 5: D2Q5 ternary 4096^2 142 / 138.7 / 142.5 / 143; D2Q9 ternary
-// 2048^2 72 / 73 / 57.5 / 67, binary 50 / 50 / 41 / 29.3; D2Q5 with four species 2048^2
-// 74.6 / 72 / 57.2 / 59.9; D2Q9 with five species 2048^2 130 / 145 / 179 (single steps:
-// 194, 86.6, 47.8, 80.5 and 180.6).
 template <int LAT, int S>
 struct RowOccupancy {
-    static constexpr int value = S >= 4 ? 2 : Lattice<LAT>::Q <= 5 ? (S == 3 ? 4 : 3) : (S == 1 ? 5 : (S == 2 ? 4 : 3));
+    static constexpr int value = row_blocks(Lattice<LAT>::Q, S);
 };
 
 // K steps of the rows [y0, y1) of one strip of W columns, with margins of H (at least K - 1).
@@ -436,13 +424,6 @@ __global__ void __launch_bounds__(kFusedBlock, 4) k_fused_line(FusedParams<S> p,
         }
 }
 
-inline f2 twice(float x)
-{
-    uint32_t b;
-    memcpy(&b, &x, 4);
-    return {((unsigned long long)b << 32) | b};
-}
-
 // Steps one fused pass may take for a solver, or 1 where none applies.  Planes: three
 // (D2Q5 ternary 4096^2: 152 us per step at two, 138 at three, 143 at four); with four or
 // five species two (their queues fill the registers).  Lines: eight (10^7 nodes: 56, 50, 47.8
@@ -456,32 +437,13 @@ constexpr int fused_limit()
     return Lattice<LAT>::DIM == 1 ? (S <= 2 ? 8 : 1) : (Lattice<LAT>::DIM == 2 && S <= 4 ? (S <= 2 ? 3 : 2) : 1);
 }
 
-// Cuts n rows into parts of at least `least` rows: `wave` parts (per strip) fill the chip
-// once.  Warps take different times, so two waves are taken while a part keeps `pair` rows
-// and up to four while it keeps `good`; but a part also forms 2 (K - 1) rows for its
-// neighbours.  D2Q5 ternary, us per step with one wave -> two: 1448^2 24.4 -> 20.4,
-// 2048 x 1100 28.5 -> 22.6, 3474 x 1576 69.5 -> 53.5 (single steps 27.7, 27.6, 65.2);
-// D2Q9 ternary 3402 x 1784 93.6 -> 86.4, but 2048^2 (31 rows) 56.5 -> 59.0, and with five
-// species, whose parts hold more, 129.9 -> 132.6.
-inline void cut(int n, double wave, int pair, int good, int least, int& segments, int& rows)
-{
-    int waves = (int)((n / good) / wave);
-    waves = waves > 4 ? 4 : waves;
-    if (waves < 2) waves = n / pair >= 2.0 * wave ? 2 : 1;
-    int s = (int)(waves * wave);
-    if (s > n / least) s = n / least;
-    if (s < 1) s = 1;
-    rows = (n + s - 1) / s;
-    segments = (n + rows - 1) / rows;
-}
-
 template <int LAT, int S, int K>
 cudaError_t launch_rows(FusedParams<S>& p, const KArgs& a)
 {
-    p.strips = (a.nx + Strip<K>::W - 1) / Strip<K>::W;
-    const double resident = (double)a.sms * RowOccupancy<LAT, S>::value * (kFusedBlock / 32);
-    constexpr int pair = Lattice<LAT>::Q <= 5 ? 16 : (S <= 2 ? 32 : 80), good = Lattice<LAT>::Q <= 5 || S <= 2 ? 48 : 80;
-    cut(a.ny, resident / p.strips, pair, good, 4 * K, p.segments, p.rows);
+    const RowPlan plan = row_plan(Lattice<LAT>::Q, S, K, a.nx, a.ny, a.sms);
+    p.strips = plan.strips;
+    p.segments = plan.segments;
+    p.rows = plan.rows;
     const uint32_t parts = (uint32_t)p.strips * (uint32_t)p.segments;
     return launch_chained(k_fused_rows<LAT, S, K>, (parts + 3) / 4, kFusedBlock, a.stream, p);
 }

@@ -439,24 +439,20 @@ cudaError_t launch_finalize(const lbms_t* h, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// Most steps one launch takes (fused.cuh): the lattice's limit on grids where a pass over
-// several steps beats as many single steps.  Times of 60-step calls, single ->
-// fused: D2Q5 ternary 1448^2 27.6 -> 24.9 us per step, 1024^2 14.0 -> 13.7 and 4096 x 300
-// 16.1 -> 16.2 (hence the higher line for it), 4096^2 194 -> 138; binary 1024^2 8.4 -> 6.0;
-// D2Q9 ternary 1024^2 23.1 -> 18.8, 724^2 11.1 -> 14.5; five species 724^2 24.3 -> 21.2;
-// lines at every length (10^4 nodes 1.80 -> 0.86, 10^6 9.6 -> 5.0).  Planes narrower than
-// two strips or lower than a few parts keep single steps, and so do grids whose planes
-// exceed 32-bit byte offsets.
+// Most steps one launch takes (fused.cuh): the lattice's limit on lines of every length (10^4
+// nodes 1.80 -> 0.86 us per step, 10^6 9.6 -> 5.0) and on planes where passes pay (rows_pay),
+// except grids whose planes exceed 32-bit byte offsets.
 int fused_depth(const lbms_t* h)
 {
     if (h->dtype != LBMS_F32 || h->relax == LBMS_RELAX_FROZEN || h->dirichlet || h->halo) return 1;
     if (h->cells >= (1u << 30)) return 1;
-    if (h->dim == 2) {
-        if (h->nx < 56 || h->ny < 24) return 1;
-        const uint32_t least = h->S >= 3 ? 1u << 19 : (h->S == 2 && h->Q <= 5 ? 3u << 19 : 1u << 20);
-        if (h->cells < least) return 1;
+    const int depth = fused_limit_of(h->lattice, h->n);
+    if (h->dim == 2 && depth > 1) {
+        const bool walls = (h->noflux & 3u) != 0;
+        const bool pairs = h->Q <= 7 && h->S <= 2 && h->cells >= kPairMinCells && (h->cells & 1u) == 0;
+        if (!rows_pay(h->Q, h->S, depth, h->nx, h->ny, walls, pairs, h->sms)) return 1;
     }
-    return fused_limit_of(h->lattice, h->n);
+    return depth;
 }
 
 // The captured graphs hold the kernel arguments: dropped whenever those change.

@@ -1,5 +1,5 @@
 // How many plain steps one launch takes, and over which parts of the grid: the rules behind
-// the passes of tile.cuh.  Plain C++, so that the host can check them.
+// the passes of tile.cuh and fused.cuh.  Plain C++, so that the host can check them.
 #pragma once
 
 namespace lbms {
@@ -75,6 +75,105 @@ inline TileShape tile_shape(int dim, int q, int s, bool f64, bool fixed, int nx,
         take(2, 8, 4, 1, 1.0) || take(2, 8, 8, 1, 0.75);
     }
     return t;
+}
+
+// The passes over rows of large FP32 planes (fused.cuh): q velocities, s evolved species.
+
+// Blocks of 4 warps per SM the row kernels are compiled for.  What bounds them is the
+// issue rate (D2Q5 ternary: 216 instructions per 32 nodes and step, of them 122 FP32, at
+// 0.75 per clock; HBM runs at 2.8 TB/s of its 6.8), so each value is the fewest warps
+// that still keep issuing, with the registers that leaves.  Measured, us per step, at
+// blocks 2 / 3 / 4 / 5: D2Q5 ternary 4096^2 142 / 138.7 / 142.5 / 143; D2Q9 ternary
+// 2048^2 72 / 73 / 57.5 / 67, binary 50 / 50 / 41 / 29.3; D2Q5 with four species 2048^2
+// 74.6 / 72 / 57.2 / 59.9; D2Q9 with five species 2048^2 130 / 145 / 179 (single steps:
+// 194, 86.6, 47.8, 80.5 and 180.6).  Ratio to the single steps, mean over planes of 1 to 4
+// million nodes: D2Q5 with five species 0.89 / 0.83 / 0.84 at 2 / 3 / 4, D2Q4 with five 0.97 / 0.91
+// / 0.91, binary D2Q4 0.93 / 0.81 / 0.98 at 3 / 4 / 5, ternary 1.08 / 1.01 / 0.94.
+constexpr int row_blocks(int q, int s)
+{
+    if (q > 5) return s == 1 ? 5 : s == 2 ? 4 : s == 3 ? 3 : 2;
+    if (q == 4 && s <= 2) return s == 1 ? 4 : 5;
+    return s == 3 ? 4 : 3;
+}
+
+// Cuts n rows into parts of at least `least` rows: `wave` parts (per strip) fill the chip
+// once.  Warps take different times, so two waves are taken while a part keeps `pair` rows
+// and up to four while it keeps `good`; but a part also forms 2 (K - 1) rows for its
+// neighbours.  D2Q5 ternary, us per step with one wave -> two: 1448^2 24.4 -> 20.4,
+// 2048 x 1100 28.5 -> 22.6, 3474 x 1576 69.5 -> 53.5 (single steps 27.7, 27.6, 65.2);
+// D2Q9 ternary 3402 x 1784 93.6 -> 86.4, but 2048^2 (31 rows) 56.5 -> 59.0, and with five
+// species, whose parts hold more, 129.9 -> 132.6.
+inline void cut(int n, double wave, int pair, int good, int least, int& segments, int& rows)
+{
+    int waves = (int)((n / good) / wave);
+    waves = waves > 4 ? 4 : waves;
+    if (waves < 2) waves = n / pair >= 2.0 * wave ? 2 : 1;
+    int s = (int)(waves * wave);
+    if (s > n / least) s = n / least;
+    if (s < 1) s = 1;
+    rows = (n + s - 1) / s;
+    segments = (n + rows - 1) / rows;
+}
+
+// The parts of a pass of `steps` steps.
+struct RowPlan {
+    int strips, segments, rows;
+};
+constexpr int row_strip(int steps) { return 32 - 2 * (steps - 1); }  // columns a warp stores
+inline double row_slots(int q, int s, int sms) { return (double)sms * row_blocks(q, s) * 4; }  // resident warps
+inline RowPlan row_plan(int q, int s, int steps, int nx, int ny, int sms)
+{
+    RowPlan p;
+    p.strips = (nx + row_strip(steps) - 1) / row_strip(steps);
+    const int pair = q <= 5 ? 16 : (s <= 2 ? 32 : 80), good = q <= 5 || s <= 2 ? 48 : 80;
+    cut(ny, row_slots(q, s, sms) / p.strips, pair, good, 4 * steps, p.segments, p.rows);
+    return p;
+}
+
+// What a pass costs: nodes formed per node of the grid (margins, idle lanes of the last
+// strip), times the warp slots per warp that has a part where the parts leave some idle; whole:
+// the slots of the last wave count as well.  At a wall along x a warp reads and selects the wall
+// nodes' own populations besides: on D2Q9 (six directions) with four and five species 0.45 and 0.6 of
+// a row's work more.
+inline double row_cost(int q, int s, int steps, int nx, int ny, bool x_walls, bool whole, int sms)
+{
+    const RowPlan p = row_plan(q, s, steps, nx, ny, sms);
+    const double waves = (double)p.strips * p.segments / row_slots(q, s, sms);
+    const double taken = whole || waves < 1.0 ? (double)(long long)(waves + 0.9999) : waves;
+    double formed = (double)p.strips * p.segments * 32.0 * (p.rows + 2 * (steps - 1)) / ((double)nx * ny);
+    if (x_walls && q > 5 && s >= 3) formed *= 1.0 + 0.15 * s * (p.strips > 1 ? 2.0 / p.strips : 1.0);
+    return formed * taken / waves;
+}
+
+// Whether passes over rows beat as many single steps.  Sizes (60-step calls, us per step,
+// single -> passes): D2Q5 ternary 1448^2 27.6 -> 24.9, 1024^2 14.0 -> 13.7 and 4096 x 300 16.1 ->
+// 16.2 (hence the higher line for it), 4096^2 194 -> 138; binary 1024^2 8.4 -> 6.0; D2Q9 ternary
+// 1024^2 23.1 -> 18.8, 724^2 11.1 -> 14.5; five species 724^2 24.3 -> 21.2; D2Q4 with four or five
+// species at 0.5 to 1 million nodes 1.0 to 1.1 times the single steps' time, at 2 million 0.9.
+// Cost: over 900 planes from 56 to 10^5 columns wide the ratio to the single steps grows with it
+// from 0.7 at 1.1, and passes 1.00 to 1.05 at the limits below; beyond them it went on to 1.2 to 1.4
+// (D2Q4 ternary 64 x 32768 20.3 -> 27.7, D2Q9 with five species 64 x 32768 91 -> 130).  pairs: the
+// grid's single steps take two nodes per thread, in three quarters of the time per node, so
+// that passes pay up to lower costs only (binary D2Q5 72 x 49498 at 1.46 22.6 -> 23.4, but 113 x
+// 18001 at 1.7 16.8 -> 14.8), and short warps feel an incomplete last wave: 66112 x 128 at 1.18 and
+// 1.29 waves 51.5 -> 61.5; with five species on D2Q9 36792 x 57 at 1.01 waves 92 -> 113.
+inline bool rows_pay(int q, int s, int steps, int nx, int ny, bool x_walls, bool pairs, int sms)
+{
+    if (s > 4 || nx < 56 || ny < 24) return false;
+    const double million = 1 << 20, cells = (double)nx * ny;
+    const double least = s >= 3 ? (q == 4 ? (s == 3 ? 1.5 : 1.0) : 0.5) : (s == 2 && q <= 5 ? 1.5 : 1.0);
+    if (cells < least * million) return false;
+    double limit;
+    if (q > 5)
+        limit = s == 1 ? 2.0 : s == 2 ? 1.7 : s == 3 ? 1.45 : 1.33;
+    else if (s == 1)
+        limit = q == 4 ? (pairs ? 1.7 : 2.05) : (pairs ? 1.42 : 1.8);
+    else if (s == 2)
+        limit = q == 4 ? 1.5 : (pairs ? 1.4 : 1.55);
+    else
+        limit = s == 3 ? 1.5 : 1.45;
+    const bool whole = (s == 1 && pairs) || (q > 5 && s >= 3);
+    return row_cost(q, s, steps, nx, ny, x_walls, whole, sms) <= limit;
 }
 
 }  // namespace lbms
