@@ -100,8 +100,18 @@ struct BatchParams {
 // The Dirichlet compositions xb ([count][6][S]) are an argument of their own:
 // inside the parameter structure the extra member changed the register
 // allocation of the kernels that do not use it.
+// FP64 binary and ternary steps keep the single solve's blocks per SM: left to itself the compiler
+// took 100 to 128 registers for ternary nodes.  us per step of 100 to 200 instances, unbounded -> 3
+// blocks: D2Q5 93.5 -> 81.4, D2Q9 120.3 -> 117.9, D3Q7 111.6 -> 102.5, binary D3Q15 90.8 -> 78.3;
+// ternary D3Q15 279 -> 219 at 2 (288 at 3).
+template <int LAT, int S, typename T>
+constexpr int batch_step_blocks()
+{
+    return sizeof(T) == 8 && S <= 2 ? StepOccupancy<LAT, S, T, true>::value : 1;
+}
+
 template <int LAT, int S, typename T, bool MASS, bool DIR>
-__global__ void __launch_bounds__(kBlock) k_batch_step(BatchParams<T> p, const T* __restrict__ xb)
+__global__ void __launch_bounds__(kBlock, batch_step_blocks<LAT, S, T>()) k_batch_step(BatchParams<T> p, const T* __restrict__ xb)
 {
     using L = Lattice<LAT>;
     constexpr int Q = L::Q;

@@ -52,3 +52,18 @@ def test_fp32_steps_leave_room_for_the_next_grid(lat, s, most, tmp_path):
     assert r.returncode == 0, r.stderr
     used = [int(v) for v in re.findall(r"Used (\d+) registers", r.stderr)]
     assert used and max(used) <= most, used
+
+
+@pytest.mark.parametrize("lat,s,blocks", [("LBMS_D2Q5", 2, 3), ("LBMS_D2Q9", 2, 3), ("LBMS_D3Q7", 2, 3), ("LBMS_D3Q15", 2, 2)])
+def test_fp64_batch_steps_keep_their_blocks_per_sm(lat, s, blocks, tmp_path):
+    """65536 registers in units of 8 per thread, blocks of 256 threads."""
+    src = tmp_path / "k.cu"
+    src.write_text('#include "batch.cuh"\nnamespace lbms {\n'
+                   "template __global__ void k_batch_step<%s, %d, double, false, false>(BatchParams<double>, "
+                   "const double*);\n}\n" % (lat, s))
+    r = subprocess.run([build.nvcc()] + build.ARCH + build.NVCC_FLAGS
+                       + ["-Xptxas", "-v", "-c", str(src), "-o", os.devnull],
+                       capture_output=True, text=True, cwd=str(tmp_path))
+    assert r.returncode == 0, r.stderr
+    used = [int(v) for v in re.findall(r"Used (\d+) registers", r.stderr)]
+    assert used and max(used) <= 65536 // (256 * blocks) // 8 * 8, used
