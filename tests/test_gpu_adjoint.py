@@ -462,3 +462,21 @@ def test_gradient_without_rest_velocity_matches_oracle_differences(lattice, dims
     fd = _fd4(lambda e: loss(D_START, x0 + e * v), 1e-4)
     ad = float((x0t.grad.cpu().numpy() * v).sum())
     assert abs(ad - fd) <= 1e-6 * abs(fd) + 1e-14, (ad, fd)
+
+
+@pytest.mark.parametrize("grid,steps", [((48, 40), 20), ((300, 300), 10)])
+def test_launch_count_of_the_forward(grid, steps):
+    """stats["launches"] counts kernels: a launch of a small grid takes several steps."""
+    from paper_1808_06787_gb300 import Solver
+    from paper_1808_06787_gb300.autograd import RunSpec, simulate
+
+    D = sy.random_D(3, seed=3)
+    s = Solver("D2Q5", D, grid)
+    K = math.ceil(math.sqrt(steps))
+    segments = [min(K, steps - t) for t in range(0, steps, K)]
+    spec = RunSpec(lattice="D2Q5", grid=grid, steps=steps)
+    x = torch.full(s.field_shape, 1.0 / 3.0, device="cuda")
+    simulate(x, torch.tensor([D[0, 1], D[0, 2], D[1, 2]], dtype=torch.float64), spec)
+    want = sum(s.step_launches(m) for m in segments)
+    assert spec.stats["launches"] == 1 + want + 1
+    assert (want < steps) == (grid == (48, 40))
