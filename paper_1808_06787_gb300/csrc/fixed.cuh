@@ -363,12 +363,11 @@ LBMS_HD bool collide_fixed(double (&f)[S][L::Q], const FixedTable& t)
         // G = k (a - c) / det K = g1 (y / 2^58) 2^(up - 3) from the scales above; q = 2 G (sum / 2)
         const X y2 = split(y << 1);
         const int64_t p1 = mul(split(half[0]), coef(mul(y2, t.g1))), p2 = mul(split(half[S - 1]), coef(mul(y2, t.g2)));
-        const int more = up > 3 ? up - 3 : 0, less = up > 3 ? 0 : 3 - up;
+        const int more = up > 3 ? up - 3 : 0;  // (det is below 2^59, so up is at least 3)
         const int64_t lim = kLimit >> more;
         fits &= p1 < lim && p1 > -lim && p2 < lim && p2 > -lim;
-        const int64_t r1 = (int64_t)((uint64_t)p1 << more) >> less, r2 = (int64_t)((uint64_t)p2 << more) >> less;
-        q1 = split(r1);
-        q2 = split(r2);
+        q1 = split((int64_t)((uint64_t)p1 << more));
+        q2 = split((int64_t)((uint64_t)p2 << more));
     }
     if (!fits) return false;
     uint64_t rest[S];  // what the moving populations leave of the sums (modulo 2^64 on the way)
@@ -474,10 +473,10 @@ __device__ __forceinline__ bool collide_fixed_lane(double (&f)[L::Q], const Fixe
         l2 = coef(mul(split(unit - h), coef(reciprocal(4 * unit - h))) >> 2);
     }
     const int64_t p = mul(split(half), coef(mul(split(y << 1), own ? t.g2 : t.g1)));
-    const int more = up > 3 ? up - 3 : 0, less = up > 3 ? 0 : 3 - up;
+    const int more = up > 3 ? up - 3 : 0;
     const int64_t lim = kLimit >> more;
     fits &= p < lim && p > -lim;
-    const X q = split((int64_t)((uint64_t)p << more) >> less);
+    const X q = split((int64_t)((uint64_t)p << more));
     const unsigned votes = __ballot_sync(all, fits);
     const int lane = (int)(threadIdx.x & 31u);
     fits = ((votes >> lane) & (votes >> (lane ^ 16)) & 1u) != 0;

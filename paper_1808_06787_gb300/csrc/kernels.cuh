@@ -614,11 +614,12 @@ __global__ void __launch_bounds__(kBlock / 2, MASS ? PairOccupancy<LAT, S, T>::m
 // (at least 2 x 2 x 3 x 4 B per node) no longer fit the 129 MB L2.
 constexpr uint32_t kPairMinCells = 1u << 21;
 
-// Largest grid stepped with two lanes per node.  us per step, one lane -> two: D2Q5 100^2
-// 3.08 -> 2.73, 128^2 3.06 -> 2.88, 200^2 4.54 -> 4.38, D2Q9 300^2 11.7 -> 10.5, D3Q7
-// 24 x 16 x 12 3.79 -> 2.61; but D2Q5 400^2 11.4 -> 11.8, 1024^2 57 -> 69, D3Q7
-// 101 x 96 x 67 47 -> 53, where the duplicated matrix work counts.
-constexpr uint32_t kSpeciesMaxCells = 3u << 15;
+// Most nodes per multiprocessor of a grid stepped with two lanes per node: beyond some twenty
+// warps per SM the duplicated matrix work counts for more than the shorter wait.  us per step at
+// 152 multiprocessors, one lane -> two: D2Q5 100^2 3.08 -> 2.73, 128^2 3.06 -> 2.88, 200^2 4.54 ->
+// 4.38, D2Q9 300^2 (592 nodes each) 11.7 -> 10.5, D3Q7 24 x 16 x 12 3.79 -> 2.61; but D2Q5 400^2
+// (1053) 11.4 -> 11.8, 1024^2 57 -> 69, D3Q7 101 x 96 x 67 47 -> 53.
+constexpr uint32_t kSpeciesNodesPerSm = 647;
 
 // Whether the pair kernel takes a step of this solver (see k_step_pair).
 template <int LAT, int S, typename T>
@@ -888,7 +889,7 @@ cudaError_t launch(Op op, const KArgs& a)
                 }
             }
             if constexpr (S == 2 && sizeof(T) == 8) {
-                if (op == OP_STEP && a.fixed.on && a.cells <= kSpeciesMaxCells)
+                if (op == OP_STEP && a.fixed.on && a.cells <= kSpeciesNodesPerSm * (uint32_t)a.sms)
                     return launch_chained(k_step_species<LAT>, (a.cells + kSmallBlock / 2 - 1) / (kSmallBlock / 2),
                                           kSmallBlock, a.stream, p);
             }

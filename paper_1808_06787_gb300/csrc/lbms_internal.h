@@ -18,8 +18,7 @@ enum Op : int {
     OP_STEP_MASS = 1,  // the same, also writing per-block mass partials
     OP_INIT = 2,       // f+ = w_k xi from a mole-fraction chunk
     OP_MOMENTS = 3,    // xi (and J) of a cell range into a field chunk
-    OP_MASS = 4,       // per-block mass partials of the current state only
-    OP_FUSED = 5       // KArgs::steps stream-collide steps fin -> fout in one pass
+    OP_MASS = 4        // per-block mass partials of the current state only
 };
 
 // A pass of several steps over tiles of a small grid (tile.cuh).
@@ -88,8 +87,9 @@ cudaError_t dispatch_halo_d1q3(Op op, int dtype, const KArgs& a);
 cudaError_t dispatch_halo_d2q4(Op op, int dtype, const KArgs& a);
 cudaError_t dispatch_halo_d3q6(Op op, int dtype, const KArgs& a);
 
-// Most steps a fused pass takes (OP_FUSED), or 1 where the solver takes single
-// steps only: per-lattice limits (kf_*.cu) within the rule of fused_depth (lbms.cu).
+// Most steps a fused pass (KArgs::steps of them, fin -> fout) takes, or 1 where the solver
+// takes single steps only: per-lattice limits (kf_planes.cu) within the rule of fused_depth
+// (lbms.cu).
 int fused_limit_of(int lattice, int n_species);
 cudaError_t dispatch_fused(int lattice, const KArgs& a);
 // A tiled pass of a.tiles.depth steps (kt_*.cu), where tile_shape (plan.h) gives one.
