@@ -164,9 +164,10 @@ def kernel_hash() -> str:
     return h.hexdigest()[:16]
 
 
-def recorded_traffic(fname: str, grid):
+def recorded_traffic(fname: str, grid, depth=None):
     """DRAM bytes per launch of a kernel from its committed ncu record, or None
-    when the kernel sources changed since it was taken or the size differs."""
+    when the kernel sources changed since it was taken or the size differs, or (depth
+    given) the recorded launch took another number of steps."""
     try:
         with open(os.path.join(ROOT, "profiles", fname)) as fh:
             rec = json.load(fh)
@@ -174,12 +175,20 @@ def recorded_traffic(fname: str, grid):
         return None
     if rec.get("kernel_hash") != kernel_hash() or list(rec.get("grid", ())) != list(grid):
         return None
+    if depth is not None and rec.get("steps_per_launch", 1) != depth:
+        return None
     return rec.get("dram_bytes_per_launch")
 
 
-def measured_traffic(wl: Workload):
+def measured_traffic(wl: Workload, depth=None):
     """DRAM bytes per launch of the workload's step kernel (see recorded_traffic)."""
-    return recorded_traffic(wl.traffic_file, wl.grid)
+    return recorded_traffic(wl.traffic_file, wl.grid, depth)
+
+
+def launch_depth(solver) -> int:
+    """Most steps one launch of a solver or batch takes: the 63 plain steps of a 64-step
+    call are split evenly over as many launches as passes of that depth need."""
+    return -(-63 // (solver.step_launches(64) - 1))
 
 
 def hbm_peak():
@@ -389,7 +398,7 @@ def measure_single(wl: Workload, steps: int, warmup: int, barrier=local_barrier,
         flags = s.status()
         mass = s.mass()
     out = {"ms": ms, "repeats_ms": reps, "status_flags": flags, "launches": s.step_launches(steps),
-           "mass_drift_rel": float(np.max(np.abs(mass - mass0) / np.abs(mass0))),
+           "depth": launch_depth(s), "mass_drift_rel": float(np.max(np.abs(mass - mass0) / np.abs(mass0))),
            "x0_host": x0_host, "stream": stream}
     if keep:
         out["solver"] = s
@@ -419,11 +428,13 @@ def single_line(wl: Workload, m: dict, steps: int, world: int, t_ms: float, sms:
     bytes_per_launch = 2.0 * wl.S * wl.Q * wl.es * wl.cells
     state_gb = bytes_per_launch / 1e9
     launches = m.get("launches", steps)  # large planes and lines take several steps per launch
+    depth = m.get("depth", 1)
     roof = (fp64_roofline(wl, t_ms / steps, sms, sm_mhz) if wl.key == "sine"
-            else hbm_roofline(bytes_per_launch, t_ms / launches, measured_traffic(wl)))
+            else hbm_roofline(bytes_per_launch, t_ms / launches, measured_traffic(wl, depth)))
     if launches < steps and wl.key != "sine":
-        roof["note"] = ("%d steps in %d launches: each reads and writes the state once; bound by the "
-                        "issue rate rather than by HBM" % (steps, launches))
+        roof["note"] = ("%d steps in %d launches: each reads and writes the state once; bound by %s "
+                        "rather than by HBM"
+                        % (steps, launches, "the FP32 pipe" if wl.key == "line" else "the issue rate"))
     return {
         "value": round(glups, 4),
         "unit": "GLUPS",
@@ -667,7 +678,7 @@ def measure_batch(steps: int, warmup: int, local: int, count: int = BATCH_COUNT,
         else:
             b.set_schedule(schedule)
             chosen, tune_ms = schedule, []
-        launches = b.step_launches(steps)
+        launches, depth = b.step_launches(steps), launch_depth(b) if chosen % 7 == 0 else 1
         x0_host = torch.empty(int(b.offsets[-1]), dtype=torch.float32).pin_memory()
         for i in range(count):
             x0_host[int(b.offsets[i]):int(b.offsets[i + 1])] = torch.from_numpy(
@@ -686,7 +697,7 @@ def measure_batch(steps: int, warmup: int, local: int, count: int = BATCH_COUNT,
     bytes_per_step = 2.0 * 2 * 5 * 4 * nodes
     passes = launches if chosen % 7 == 0 else steps
     roof = hbm_roofline(bytes_per_step, ms / passes,
-                        recorded_traffic("traffic_batch_d2q5_4096_f32.json", [count, int(chosen)])
+                        recorded_traffic("traffic_batch_d2q5_4096_f32.json", [count, int(chosen)], depth)
                         if chosen % 7 == 0 else None)
     roof["note"] = ("algorithmic bytes of a streamed launch (%d steps in %d launches); L2-blocked "
                     "schedules move less" % (steps, passes))

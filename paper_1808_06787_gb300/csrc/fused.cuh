@@ -21,7 +21,7 @@
 #include <type_traits>
 
 #include "kernels.cuh"
-#include "plan.h"
+#include "plan.cuh"
 
 namespace lbms {
 
@@ -87,7 +87,7 @@ struct March {
 constexpr int kFusedBlock = 128;
 
 // Rows of a plane (2D).  A lane owns one column of its warp's strip of 32 columns, K - 1 of
-// them on each side only to feed the later steps (row_plan, plan.h).
+// them on each side only to feed the later steps (row_plan, plan.cuh).
 
 // The grid a warp marches through: a plane of its own, or one of a batch's (whose nodes
 // begin at `base` of a common node space).

@@ -13,7 +13,7 @@
 #include "adjoint.cuh"
 #include "lbms_internal.h"
 #include "node.cuh"
-#include "plan.h"
+#include "plan.cuh"
 
 using namespace lbms;
 

@@ -92,7 +92,7 @@ cudaError_t dispatch_halo_d3q6(Op op, int dtype, const KArgs& a);
 // (lbms.cu).
 int fused_limit_of(int lattice, int n_species);
 cudaError_t dispatch_fused(int lattice, const KArgs& a);
-// A tiled pass of a.tiles.depth steps (kt_*.cu), where tile_shape (plan.h) gives one.
+// A tiled pass of a.tiles.depth steps (kt_*.cu), where tile_shape (plan.cuh) gives one.
 cudaError_t dispatch_tile(int lattice, int dtype, const KArgs& a);
 template <int LAT>
 cudaError_t dispatch_tile_lattice(int dtype, const KArgs& a);

@@ -112,3 +112,26 @@ def test_sharded_grid_stacks_one_workload_grid_per_rank():
     assert bench.sharded_grid(bench.make_workload("blobs", 256), 2) == (2048, 4096, 1)
     assert bench.sharded_grid(bench.make_workload("line", 256), 8) == (8 << 26, 1, 1)
     assert bench.sharded_grid(bench.make_workload("tube", 256), 1) == (256, 256, 256)
+
+
+def test_traffic_record_needs_the_depth_of_the_timed_launches(tmp_path, monkeypatch):
+    rec = {"kernel_hash": "abc123", "grid": [8, 8, 1], "steps_per_launch": 2, "dram_bytes_per_launch": 7.0}
+    (tmp_path / "profiles").mkdir()
+    (tmp_path / "profiles" / "t.json").write_text(json.dumps(rec))
+    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+    monkeypatch.setattr(bench, "kernel_hash", lambda: "abc123")
+    assert bench.recorded_traffic("t.json", (8, 8, 1), 2) == 7.0
+    assert bench.recorded_traffic("t.json", (8, 8, 1), 3) is None
+    rec.pop("steps_per_launch")  # single steps
+    (tmp_path / "profiles" / "t.json").write_text(json.dumps(rec))
+    assert bench.recorded_traffic("t.json", (8, 8, 1), 1) == 7.0
+    assert bench.recorded_traffic("t.json", (8, 8, 1), 3) is None
+
+
+@pytest.mark.parametrize("depth", [1, 2, 3, 4, 5, 8])
+def test_launch_depth(depth):
+    class Fake:
+        def step_launches(self, n):
+            return 1 + -(-(n - 1) // depth)
+
+    assert bench.launch_depth(Fake()) == depth

@@ -1,4 +1,4 @@
-"""The rules that choose passes of several steps (plan.h), compiled for the host.
+"""The rules that choose passes of several steps (plan.cuh), compiled for the host.
 
 Tiles: whatever the grid's shape, a launch forms a bounded number of nodes per
 multiprocessor and step; a grid of few nodes but many tiles (one node wide, or flat) takes
@@ -21,7 +21,7 @@ ROOT = os.path.dirname(HERE)
 SMS = 152
 
 SOURCE = r"""
-#include "plan.h"
+#include "plan.cuh"
 extern "C" int tiles(int dim, int q, int s, int f64, int fixed, int nx, int ny, int nz, int sms, int* out)
 {
     const lbms::TileShape t = lbms::tile_shape(dim, q, s, f64 != 0, fixed != 0, nx, ny, nz, sms);
