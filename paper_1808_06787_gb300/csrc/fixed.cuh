@@ -8,8 +8,8 @@
 // error (rms 0.9e-16 of a population against 1.8e-16).  Measured, us per step, FP64 ->
 // fixed point: ternary D2Q5 128^2 5.77 -> 3.02, 200^2 12.35 -> 4.48, 1024^2 232 -> 56;
 // D3Q7 101 x 96 x 67 189 -> 45.5; D2Q9 300^2 42 -> 11.4; binary D2Q5 240 x 40 3.18 -> 1.87.
-// The large grids are bound by the integer and FP64 pipes together (59 % and 75 %), the
-// small ones by the latency of a step.
+// The large grids are bound by the integer and FP64 pipes together (D3Q7 101 x 96 x 67: ALU 69 %,
+// FP64 50 % busy, 64 % of the issue slots), the small ones by the latency of a step.
 //
 //   populations  each species' populations at a node are integers X in units of 2^-58 of
 //                the power of two above the largest of them (a block exponent M), so a

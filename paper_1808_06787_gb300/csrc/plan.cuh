@@ -80,9 +80,10 @@ inline TileShape tile_shape(int dim, int q, int s, bool f64, bool fixed, int nx,
 // The passes over rows of large FP32 planes (fused.cuh): q velocities, s evolved species.
 
 // Blocks of 4 warps per SM the row kernels are compiled for.  What bounds them is the
-// issue rate (D2Q5 ternary: 216 instructions per 32 nodes and step, of them 122 FP32, at
-// 0.75 per clock; HBM runs at 2.8 TB/s of its 6.8), so each value is the fewest warps
-// that still keep issuing, with the registers that leaves.  Measured, us per step, at
+// issue rate (D2Q5 ternary 2048^2: 265 instructions per 32 nodes stored and step, margins
+// included, in 78 % of the issue slots, the FP32 pipes 49 % and the ALU 46 % busy; HBM runs at 2.7
+// TB/s of its 6.8), so each value is the fewest warps that still keep issuing, with the
+// registers that leaves.  Measured, us per step, at
 // blocks 2 / 3 / 4 / 5: D2Q5 ternary 4096^2 142 / 138.7 / 142.5 / 143; D2Q9 ternary
 // 2048^2 72 / 73 / 57.5 / 67, binary 50 / 50 / 41 / 29.3; D2Q5 with four species 2048^2
 // 74.6 / 72 / 57.2 / 59.9; D2Q9 with five species 2048^2 130 / 145 / 179 (single steps:
