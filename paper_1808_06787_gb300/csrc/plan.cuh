@@ -2,6 +2,8 @@
 // the passes of tile.cuh and fused.cuh.  Plain C++, so that the host can check them.
 #pragma once
 
+#include <initializer_list>
+
 namespace lbms {
 
 // Tile of a pass over a small grid (tile.cuh) and the most steps it takes; depth 1: single
@@ -10,6 +12,14 @@ struct TileShape {
     int depth;
     int x, y, z;
 };
+
+// Nodes of a 2D tile and its margins that a step of its pass forms, on average over the steps.
+inline double tile_formed(const TileShape& t)
+{
+    double sum = 0.0;
+    for (int m = 0; m < t.depth; ++m) sum += (double)(t.x + 2 * m) * (t.y + 2 * m);
+    return sum / t.depth;
+}
 
 inline double tile_count(const TileShape& t, int nx, int ny, int nz)
 {
@@ -28,6 +38,10 @@ inline double tile_count(const TileShape& t, int nx, int ny, int nz)
 // grid of 8192 x 1 (1024 of 8 x 8) it was 1.87 -> 2.37, of 65536 x 1 (4096 of 16 x 16) 2.27 ->
 // 17.2, of D2Q9's 4096 x 2 (256 of 16 x 16) 2.07 -> 2.18.  Four species fill an SM with one
 // tile of 16 x 16: D2Q9 158 x 186 (120 tiles) 2.64 -> 2.37 and 204^2 (169 tiles) 2.77 -> 3.87.
+// Grids of more tiles, flat ones above all, take passes while a step's work, the nodes formed
+// times S Q + 4 (about the instructions of a node), is at most 7900 per multiprocessor: binary
+// D2Q5 6000 x 4 (4700) 1.97 -> 1.19, 5000 x 13 (6100) 2.06 -> 1.65, ternary 6000 x 4 (7400) 1.97 ->
+// 1.81, but D2Q9 4096 x 2 (12100 in tiles of 16 x 16) 2.07 -> 2.18.
 // FP32 volumes: D3Q7 24 x 16 x 12 1.79 -> 1.33, 28 x 24 x 16 1.95 -> 1.63, 40 x 24 x 24 2.08 -> 2.10
 // (single); 7168 x 1 x 1 (1792 tiles of 4^3) 1.97 -> 10.7.
 // FP64 in fixed point: binary D2Q5 240 x 40 1.79 -> 1.22, 128^2 1.78 -> 1.44, ternary 64^2 2.84
@@ -51,7 +65,6 @@ inline TileShape tile_shape(int dim, int q, int s, bool f64, bool fixed, int nx,
         t = c;
         return true;
     };
-    const double nodes = (double)nx * ny * nz;
     if (s > 3 || (f64 && s > 2)) return none;
     if (dim == 1) {
         take(8, 16, 1, 1, 3.375);
@@ -59,18 +72,27 @@ inline TileShape tile_shape(int dim, int q, int s, bool f64, bool fixed, int nx,
         if (f64 || s > 2 || q > 7) return none;
         take(3, 4, 4, 4, 0.75) || take(2, 8, 4, 4, 1.0);
     } else if (!f64) {
-        if (take(5, 8, 8, 1, 1.0) || take(4, 16, 8, 1, 1.4)) return t;
+        const double nodes = (double)nx * ny;
+        if (take(5, 8, 8, 1, 1.0) || (nodes <= 162.0 * sms && take(4, 16, 8, 1, 1.65))) return t;
         // two waves of the largest tiles cost as much however few nodes they hold
-        if (nodes < 128.0 * tile_count({1, 16, 16, 1}, nx, ny, nz)) return none;
-        if (s == 2 && q <= 5 && take(2, 16, 16, 1, 1.8, 1.05)) return t;
-        take(3, 16, 16, 1, s == 3 ? 1.0 : 1.8);
+        if (nodes >= 128.0 * tile_count({1, 16, 16, 1}, nx, ny, nz)) {
+            if (s == 2 && q <= 5 && take(2, 16, 16, 1, 1.8, 1.12)) return t;
+            if (take(3, 16, 16, 1, s == 3 && q > 5 ? 1.0 : 1.8)) return t;
+        }
+        double least = 7900.0 * sms;
+        for (const TileShape& c : {TileShape{5, 8, 8, 1}, TileShape{4, 16, 8, 1}, TileShape{3, 16, 16, 1}}) {
+            const double work = tile_count(c, nx, ny, nz) * tile_formed(c) * (s * q + 4);
+            if (work > least) continue;
+            least = work;
+            t = c;
+        }
     } else if (fixed) {
         if (s == 1)
             take(5, 8, 8, 1, 1.0) || take(4, 16, 8, 1, 1.1);
         else
             take(4, 8, 4, 1, 0.9) || take(5, 8, 8, 1, 0.75);
     } else if (s == 1) {
-        take(2, 8, 4, 1, 1.0) || take(2, 8, 8, 1, 1.0) || (nodes > 128.0 * sms && take(2, 12, 12, 1, 1.0, 0.9));
+        take(2, 8, 4, 1, 1.0) || take(2, 8, 8, 1, 1.0) || ((double)nx * ny > 128.0 * sms && take(2, 12, 12, 1, 1.0, 0.9));
     } else {
         take(2, 8, 4, 1, 1.0) || take(2, 8, 8, 1, 0.75);
     }
