@@ -415,8 +415,9 @@ long plain_launches(const lbms_t* h, long n, bool replay = false)
 }
 
 // n plain steps from f[src], split evenly over the passes (so that none is left a
-// single step where it can be helped); src becomes the buffer that holds the result.
-cudaError_t launch_plain(const lbms_t* h, int& src, long n, cudaStream_t st, bool replay = false)
+// single step where it can be helped); src becomes the buffer that holds the result and n the
+// steps not taken (of a launch that failed, and those after it).
+cudaError_t launch_plain(const lbms_t* h, int& src, long& n, cudaStream_t st, bool replay = false)
 {
     for (long passes = plain_launches(h, n, replay); passes > 0; --passes) {
         const int m = (int)((n + passes - 1) / passes);
@@ -476,7 +477,8 @@ cudaError_t build_call_graph(lbms_t* h, long n, int parity, cudaGraphExec_t* out
     cudaError_t e = cudaStreamBeginCapture(h->capture, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
     int src = parity;
-    cudaError_t le = launch_plain(h, src, n - 1, h->capture);
+    long plain = n - 1;
+    cudaError_t le = launch_plain(h, src, plain, h->capture);
     if (le == cudaSuccess) le = launch_step(h, src, true, h->capture);
     cudaGraph_t g = nullptr;
     e = cudaStreamEndCapture(h->capture, &g);
@@ -521,7 +523,8 @@ cudaError_t build_graph(lbms_t* h, int parity, int j)
     cudaError_t e = cudaStreamBeginCapture(h->capture, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
     int src = parity;
-    cudaError_t le = launch_plain(h, src, kGraphLens[j], h->capture);
+    long plain = kGraphLens[j];
+    cudaError_t le = launch_plain(h, src, plain, h->capture);
     cudaGraph_t g = nullptr;
     e = cudaStreamEndCapture(h->capture, &g);
     if (le != cudaSuccess) {
@@ -876,10 +879,11 @@ int lbms_step(lbms_t* h, long n_steps)
     }
     while (left > 1) {
         const long m = left - 1 < kCallGraphMax ? left - 1 : kCallGraphMax;
-        e = launch_plain(h, h->cur, m, h->stream, captured);
+        long rest = m;
+        e = launch_plain(h, h->cur, rest, h->stream, captured);
+        left -= m - rest;
+        h->steps += m - rest;
         if (e != cudaSuccess) return cuda_fail(h, e, "step kernel");
-        left -= m;
-        h->steps += m;
     }
     e = launch_step(h, h->cur, true, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "step kernel");
